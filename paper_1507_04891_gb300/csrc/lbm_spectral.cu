@@ -1271,12 +1271,20 @@ struct GraphStatus {
   int need[4];         // steps that needed 1, 2, 3, >= 4 applications since the host reset it
   int needf[4];        // the same, counting only steps whose start had the full history
   int full;            // the current step's start had the full history
-  double start_log;    // sum of log10 of the steps' start residuals
-  long long starts;    // steps counted in start_log
+  // product of the squares of the steps' start residuals, start_mant (in
+  // [1, 2)) times 2^start_exp
+  double start_mant;
+  long long start_exp;
+  long long starts;    // steps counted in the product
   int spec_skip;       // the current step does not speculate (start from a short history)
   long long redos;     // steps that ran the stream/collide after the loop
   int more;            // the first test of the step asks for more applications
 };
+
+// Sum of log10 of the steps' start residuals.
+double start_log(const GraphStatus& g) {
+  return 0.5 * (log10(g.start_mant) + (double)g.start_exp * 0.30102999566398119521);
+}
 
 // First node of the rerun branch: the loop runs when the step's first test
 // asked for more applications (it reruns the stream/collide also when the
@@ -1298,51 +1306,69 @@ __global__ void k_spec_decide(const int* __restrict__ start_terms, GraphStatus* 
   st->spec_skip = ((start_terms && *start_terms < START_FULL_TERMS) || st->iters > k) ? 1 : 0;
 }
 
-// Convergence test (one warp).  first: after the k applications queued
-// unconditionally (norm slots 0..k hold the residual before each and after
-// the last); records how many a step needed and sets `redo` when the loop
-// will run.  Otherwise after one more application (slot k).  Sets the
-// condition of the while node.
-__global__ void k_graph_check(const float* __restrict__ acc, GraphStatus* st, double tol,
-                              double floor2, int maxit, int k, int first,
-                              const int* __restrict__ start_terms,
-                              cudaGraphConditionalHandle cond, cudaGraphConditionalHandle redo) {
-  if (blockIdx.x != 0) return;
-  const int lane = threadIdx.x;
-  // lane i < k + 1 tests slot i
-  bool conv_i = false;
-  double rn2 = 0.0, sn2 = 0.0;
-  if (lane <= k) {
-    const float* a = acc + (size_t)lane * 2 * NACC;
-    for (int j = 0; j < NACC; ++j) {
-      rn2 += (double)a[j];
-      sn2 += (double)a[NACC + j];
+// Convergence test (one CTA, one warp per norm slot).  first: after the k
+// applications queued unconditionally (norm slots 0..k hold the residual
+// before each and after the last); records how many a step needed and sets
+// `redo` when the loop will run.  Otherwise after one more application (slot
+// k).  Sets the condition of the while node.
+//
+// Latency-bound, on the step's critical path for small lattices (beside the
+// stream/collide for large ones).  Warp i sums slot i: four loads in flight
+// per lane and FP64 shuffles, and the divisions and the square root of the
+// first and the last slot run in different warps.  One lane per slot that
+// walked its 128 values in FP64 took 14.0 us a step on a 32x8x52 slit and
+// 16.1 us on a 64x64x66 one; this form is 4.3 and 6.9 us.  The start
+// residuals are accumulated as a product (mantissa and exponent, so that no
+// logarithm is evaluated here).
+__global__ void __launch_bounds__(32 * Poisson::NSLOT)
+    k_graph_check(const float* __restrict__ acc, GraphStatus* st, double tol, double floor2,
+                  int maxit, int k, int first, const int* __restrict__ start_terms,
+                  cudaGraphConditionalHandle cond, cudaGraphConditionalHandle redo) {
+  __shared__ int conv_s[Poisson::NSLOT];
+  const int lane = threadIdx.x & 31, slot = threadIdx.x >> 5;
+  static_assert(NACC == 64, "two values of each norm per lane");
+  {
+    const float* a = acc + (size_t)slot * 2 * NACC;
+    const float r0 = a[lane], r1 = a[lane + 32], s0 = a[NACC + lane], s1 = a[NACC + lane + 32];
+    double rn2 = (double)r0 + (double)r1, sn2 = (double)s0 + (double)s1;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      rn2 += __shfl_xor_sync(0xffffffffu, rn2, off);
+      sn2 += __shfl_xor_sync(0xffffffffu, sn2, off);
     }
     rn2 *= 1099511627776.0;
     sn2 *= 1099511627776.0;
-    conv_i = rn2 <= tol * tol * sn2 || rn2 <= floor2;
+    if (lane == 0) {
+      conv_s[slot] = rn2 <= tol * tol * sn2 || rn2 <= floor2;
+      if (slot == k) st->rel = sn2 > 0.0 ? sqrt(rn2 / sn2) : 0.0;
+    } else if (lane == 1 && slot == 0 && first && rn2 >= 0.0 && sn2 > 0.0) {
+      // slot 0 holds the residual the first application transformed (the
+      // start); the product's exponent goes to start_exp
+      const double m = st->start_mant * fmax(rn2 / sn2, 1e-290);
+      const long long b = __double_as_longlong(m);
+      st->start_exp += ((b >> 52) & 0x7ff) - 1023;
+      st->start_mant = __longlong_as_double((b & 0x800fffffffffffffLL) | (1023LL << 52));
+      st->starts += 1;
+    }
   }
-  const unsigned convmask = __ballot_sync(0xffffffffu, conv_i);
-  const double rnk = __shfl_sync(0xffffffffu, rn2, k), snk = __shfl_sync(0xffffffffu, sn2, k);
-  if (lane != 0) return;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  unsigned convmask = 0;
+  for (int i = 0; i <= k; ++i) convmask |= conv_s[i] ? 1u << i : 0u;
   const bool conv = (convmask >> k) & 1u;
   // the step counts towards the choice of k when its start was near the
   // one of the steady state: fitted on at least START_FULL_TERMS stored
   // differences (the first starts after a restart have fewer), or any step
   // when the history start is off
+  int iters;
   if (first) {
     st->full = !start_terms || *start_terms >= START_FULL_TERMS;
-    st->iters = k;
-    // slot 0 holds the residual the first application transformed (the
-    // start), lane 0 read it
-    if (rn2 >= 0.0 && sn2 > 0.0) {
-      st->start_log += 0.5 * log10(fmax(rn2 / sn2, 1e-300));
-      st->starts += 1;
-    }
+    iters = k;
   } else {
-    st->iters += 1;
+    iters = st->iters + 1;
   }
-  const bool more = !conv && st->iters < maxit;
+  st->iters = iters;
+  const bool more = !conv && iters < maxit;
   // the stream/collide ran beside this test on the potential after k
   // applications: it runs again after the loop when the loop runs, or when
   // the step did not speculate.  The first test opens that branch (its loop
@@ -1356,7 +1382,6 @@ __global__ void k_graph_check(const float* __restrict__ acc, GraphStatus* st, do
   } else {
     cudaGraphSetConditional(cond, more ? 1u : 0u);
   }
-  st->rel = snk > 0.0 ? sqrt(rnk / snk) : 0.0;
   // applications this step needed, recorded once per step: at the first
   // test when slot k converged (the earliest converged slot), else when the
   // loop ends
@@ -1364,14 +1389,14 @@ __global__ void k_graph_check(const float* __restrict__ acc, GraphStatus* st, do
   if (first && conv)
     needed = max(1, __ffs(convmask) - 1);
   else if (!more)
-    needed = st->iters;
+    needed = iters;
   if (needed) {
     const int j = min(needed, 4) - 1;
     st->need[j] += 1;
     if (st->full) st->needf[j] += 1;
   }
   if (!more) {
-    st->total += st->iters;
+    st->total += iters;
     if (!conv) st->fails += 1;
   }
 }
@@ -1489,7 +1514,7 @@ lbm_status build_step_graph(lbm_t* h, int parity, bool diag) {
     if (ec == cudaSuccess) ec = cudaEventRecord(join, side);
     if (ec == cudaSuccess) ec = spec_residual(h, k, false);
     if (ec == cudaSuccess) {
-      k_graph_check<<<1, 32, 0, main>>>(norm_slot(h, 0), gs, tol, floor2, maxit, k, 1, terms, cond,
+      k_graph_check<<<1, 32 * (k + 1), 0, main>>>(norm_slot(h, 0), gs, tol, floor2, maxit, k, 1, terms, cond,
                                         redo);
       ++h->launches;
       ec = cudaGetLastError();
@@ -1563,7 +1588,7 @@ lbm_status build_step_graph(lbm_t* h, int parity, bool diag) {
         cudaError_t eb = spec_apply(h, 0);
         if (eb == cudaSuccess) eb = spec_residual(h, k, false);
         if (eb == cudaSuccess) {
-          k_graph_check<<<1, 32, 0, main>>>(norm_slot(h, 0), gs, tol, floor2, maxit, k, 0, terms,
+          k_graph_check<<<1, 32 * (k + 1), 0, main>>>(norm_slot(h, 0), gs, tol, floor2, maxit, k, 0, terms,
                                             cond, redo);
           ++h->launches;
           eb = cudaGetLastError();
@@ -1665,6 +1690,7 @@ lbm_status spectral_graph_steps(lbm_t* h, int nsteps) {
     }
     GraphStatus z = {};
     z.step = (uint32_t)h->tstep;
+    z.start_mant = 1.0;
     cudaMemcpy(p, &z, sizeof z, cudaMemcpyHostToDevice);
     h->gstatus = p;
     if (cudaMallocHost(&h->hstatus, sizeof(GraphStatus)) != cudaSuccess) {
@@ -1688,7 +1714,7 @@ lbm_status spectral_graph_steps(lbm_t* h, int nsteps) {
   LBM_CUDA_TRY(h, charge_prepare(h));
   const long long total0 = hs->total;
   const int fails0 = hs->fails;
-  const double slog0 = hs->start_log;
+  const double slog0 = start_log(*hs);
   const long long starts0 = hs->starts;
   // Steps are replayed in chunks.  The distribution of the applications
   // the steps needed (accumulated over at least CHUNK steps whose start had
@@ -1785,7 +1811,7 @@ lbm_status spectral_graph_steps(lbm_t* h, int nsteps) {
   if (hs->starts > starts0) {
     // start residuals of the replayed steps (their geometric mean stands
     // for the last one)
-    const double dl = hs->start_log - slog0;
+    const double dl = start_log(*hs) - slog0;
     const long long dn = hs->starts - starts0;
     h->start_log_sum += dl;
     h->start_count += dn;
