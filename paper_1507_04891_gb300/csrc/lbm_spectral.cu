@@ -613,117 +613,197 @@ __global__ void k_global_mean(const double* dsum, double inv_nfluid, long long* 
 // x at the first plane of the run is pinned to 0 and the remaining planes
 // are solved (the pinned plane's equation is redundant once the run sum of
 // the right-hand side is zero, which the run-mean removal guarantees).
-// X, C, Qv: the pencil's values, elimination factors and the Sherman-
-// Morrison auxiliary vector, element k at index k * st (shared memory).
 struct Run {
   int z0, len, cyclic;
 };
 
-__device__ void solve_pencil(float2* X, float* C, float* Qv, int st, int L, float lam,
-                             bool singular, bool cyclic) {
-  auto thomas = [&](int k0, int k1, auto diagf, bool with_q, auto qrhs) {
-    // forward elimination on planes k0..k1-1 (off-diagonals -1)
-    float c = 0.f, dq = 0.f;
-    float2 d = make_float2(0.f, 0.f);
-    for (int k = k0; k < k1; ++k) {
-      const float den = diagf(k) + (k > k0 ? c : 0.f);
-      const float inv = 1.0f / den;
-      const float2 rk = X[k * st];
-      d = make_float2((rk.x + (k > k0 ? d.x : 0.f)) * inv, (rk.y + (k > k0 ? d.y : 0.f)) * inv);
-      if (with_q) {
-        dq = (qrhs(k) + (k > k0 ? dq : 0.f)) * inv;
-        Qv[k * st] = dq;
-      }
-      c = -inv;
-      X[k * st] = d;
-      C[k * st] = c;
+constexpr int ZP = 32;  // pencils (Fourier modes) per CTA of the z solve
+
+// Elimination factors of the z solve, the same for every solve of a plan:
+// row k of mode m eliminates with inv = 1 / (diagonal - inv_{k-1}), which
+// depends on the mode and k only, except in a run's last row (its diagonal
+// knows the end; the solve forms that one).  tab[k mxy + m], k < len.
+// cyclic (one run, the whole periodic axis): Sherman-Morrison
+// A = T + u v^T with corners -1, gamma = -b, b = lambda + 2,
+// T = A without corners, T_00 = b - gamma, T_LL = b - 1/gamma,
+// u = (gamma, 0, .., 0, -1), v = (1, 0, .., 0, -1/gamma): the factors of T
+// (every row) and qtab = T^-1 u.
+__global__ void __launch_bounds__(128) k_ztable(float* __restrict__ tab, float* __restrict__ qtab,
+                                                int len, int cyclic, SpecArgs a) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= a.mxy) return;
+  const int ky = m / (a.H + 1), kx = m - ky * (a.H + 1);
+  const float lam = a.lamx[kx] + a.lamy[ky];
+  const int64_t mxy = a.mxy;
+  const bool singular = m == 0;
+  const int k0 = singular ? 1 : 0;
+  if (singular) tab[m] = 0.f;
+  const float b = lam + 2.f, gam = -b;
+  float c = 0.f, dq = 0.f;
+  for (int k = k0; k < len; ++k) {
+    float diag;
+    if (singular) diag = 2.f;
+    else if (cyclic) diag = k == 0 ? b - gam : (k == len - 1 ? b - 1.0f / gam : b);
+    else diag = lam + (k > 0 ? 2.f : 1.f);
+    const float inv = 1.0f / (diag + (k > k0 ? c : 0.f));
+    tab[k * mxy + m] = inv;
+    c = -inv;
+    if (cyclic && !singular) {
+      const float u = k == 0 ? gam : (k == len - 1 ? -1.f : 0.f);
+      dq = (u + (k > 0 ? dq : 0.f)) * inv;
+      qtab[k * mxy + m] = dq;
     }
-    float2 nx_ = X[(k1 - 1) * st];
-    float nq = with_q ? Qv[(k1 - 1) * st] : 0.f;
-    for (int k = k1 - 2; k >= k0; --k) {
-      const float ck = C[k * st];
-      const float2 dk = X[k * st];
-      nx_ = make_float2(dk.x - ck * nx_.x, dk.y - ck * nx_.y);
-      X[k * st] = nx_;
-      if (with_q) {
-        nq = Qv[k * st] - ck * nq;
-        Qv[k * st] = nq;
-      }
-    }
-  };
-  auto noq = [](int) { return 0.f; };
-  if (!cyclic) {
-    auto diag = [&](int k) { return lam + (float)((k > 0) + (k < L - 1)); };
-    if (singular) {
-      X[0] = make_float2(0.f, 0.f);
-      if (L > 1) thomas(1, L, diag, false, noq);
-    } else {
-      thomas(0, L, diag, false, noq);
-    }
-    return;
   }
-  if (singular) {
-    // pin x_0 = 0; planes 1..L-1 form a Dirichlet chain (diagonal 2)
-    X[0] = make_float2(0.f, 0.f);
-    thomas(1, L, [](int) { return 2.f; }, false, noq);
-    return;
-  }
-  // Sherman-Morrison: A = T + u v^T, corners -1, gamma = -b,
-  // T = A without corners, T_00 = b - gamma, T_LL = b - 1/gamma,
-  // u = (gamma, 0, .., 0, -1), v = (1, 0, .., 0, -1/gamma).
-  const float b = lam + 2.f;
-  const float gam = -b;
-  auto tdiag = [&](int k) {
-    return k == 0 ? b - gam : (k == L - 1 ? b - 1.0f / gam : b);
-  };
-  auto urhs = [&](int k) { return k == 0 ? gam : (k == L - 1 ? -1.f : 0.f); };
-  thomas(0, L, tdiag, true, urhs);
-  const float2 y0 = X[0], yl = X[(L - 1) * st];
-  const float q0 = Qv[0], ql = Qv[(L - 1) * st];
-  const float den = 1.f + q0 - ql / gam;
-  const float2 f = make_float2((y0.x - yl.x / gam) / den, (y0.y - yl.y / gam) / den);
-  for (int k = 0; k < L; ++k) {
-    const float qk = Qv[k * st];
-    const float2 yk = X[k * st];
-    X[k * st] = make_float2(yk.x - qk * f.x, yk.y - qk * f.y);
+  if (cyclic && !singular) {
+    float nq = dq;
+    for (int k = len - 2; k >= 0; --k) {
+      nq = fmaf(tab[k * mxy + m], nq, qtab[k * mxy + m]);
+      qtab[k * mxy + m] = nq;
+    }
+  } else if (cyclic) {
+    for (int k = 0; k < len; ++k) qtab[k * mxy + m] = 0.f;
   }
 }
 
-constexpr int ZP = 32;  // pencils (Fourier modes) per CTA of the z solve
+// One CTA: ZP consecutive modes of one run.  The pencils and their
+// elimination factors are staged in shared memory (coalesced: consecutive
+// modes are contiguous in each plane), solved one per thread of the first
+// warp, and written back in place.  Latency-bound: with the factors from
+// the table a row costs one add and one multiply forward and one FMA
+// backward, its operands loaded ZB rows ahead, where forming the factor cost
+// a division per row in the chain (32x8x52 slit: 13.5 -> 4.0 us; 64x64x66
+// slit: 18.4 -> 7 us; 64 slits of 32x32: 53 -> 24 us).
+constexpr int ZB = 8;
 
-// One CTA: ZP consecutive modes of one run.  The pencils are staged in
-// shared memory (coalesced: consecutive modes are contiguous in each
-// plane), solved one per thread, and written back in place.
-__global__ void __launch_bounds__(128) k_zsolve(float2* __restrict__ x,
+constexpr int ZT = 256;  // threads of a CTA: rows staged ZT / ZP at a time
+
+__global__ void __launch_bounds__(ZT) k_zsolve(float2* __restrict__ x,
                                                 const Run* __restrict__ runs,
-                                                SpecArgs a) {
-  extern __shared__ float zsm[];
+                                                const float* __restrict__ tab,
+                                                const float* __restrict__ qtab, SpecArgs a) {
+  extern __shared__ __align__(16) float zsm[];
+  __shared__ float2 fs[ZP];
   const Run R = runs[blockIdx.y];
   const int L = R.len;
-  const int nxy = a.mxy;  // modes per plane of the half spectrum
+  const int64_t nxy = a.mxy;  // modes per plane of the half spectrum
   const int m0 = blockIdx.x * ZP;
   float2* X = reinterpret_cast<float2*>(zsm);
-  float* C = zsm + 2 * ZP * L;
-  float* Qv = C + ZP * L;
-  for (int idx = threadIdx.x; idx < ZP * L; idx += blockDim.x) {
-    const int k = idx / ZP, j = idx - k * ZP;
-    int z = R.z0 + k;
-    if (z >= a.nz) z -= a.nz;
-    if (m0 + j < nxy) X[idx] = x[(int64_t)z * nxy + m0 + j];
+  float* V = zsm + 2 * ZP * L;
+  const int j = threadIdx.x & (ZP - 1), kk = threadIdx.x / ZP;
+  constexpr int KT = ZT / ZP;
+  const bool ok = m0 + j < a.mxy;
+  if (ok) {
+    for (int kb = kk; kb < L; kb += ZB * KT) {
+      float2 r[ZB];
+      float v[ZB];
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) {
+        const int k = min(kb + u * KT, L - 1);  // past the run: a repeat, unused
+        int z = R.z0 + k;
+        if (z >= a.nz) z -= a.nz;
+        r[u] = x[z * nxy + m0 + j];
+        v[u] = __ldg(tab + k * nxy + m0 + j);
+      }
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) {
+        const int k = kb + u * KT;
+        if (k < L) {
+          X[k * ZP + j] = r[u];
+          V[k * ZP + j] = v[u];
+        }
+      }
+    }
   }
   __syncthreads();
-  const int j = threadIdx.x;
-  if (j < ZP && m0 + j < nxy) {
+  if (threadIdx.x < ZP && ok) {
     const int m = m0 + j;
     const int ky = m / (a.H + 1), kx = m - ky * (a.H + 1);
-    solve_pencil(X + j, C + j, Qv + j, ZP, L, a.lamx[kx] + a.lamy[ky], m == 0, R.cyclic != 0);
+    const float lam = a.lamx[kx] + a.lamy[ky];
+    float2* Xp = X + j;
+    float* Vp = V + j;
+    const bool singular = m == 0;
+    const int k0 = singular ? 1 : 0;
+    if (!R.cyclic && L - 1 >= k0) {
+      // the last row of a run between walls: one open face
+      const float diag = singular ? 1.f : lam + (L > 1 ? 1.f : 0.f);
+      const float c = L - 1 > k0 ? -Vp[(L - 2) * ZP] : 0.f;
+      Vp[(L - 1) * ZP] = 1.0f / (diag + c);
+    }
+    if (singular) Xp[0] = make_float2(0.f, 0.f);
+    // forward elimination (off-diagonals -1)
+    float2 d = make_float2(0.f, 0.f);
+    int k = k0;
+    for (; k + ZB <= L; k += ZB) {
+      float2 r[ZB];
+      float v[ZB];
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) {
+        r[u] = Xp[(k + u) * ZP];
+        v[u] = Vp[(k + u) * ZP];
+      }
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) {
+        d = make_float2((r[u].x + d.x) * v[u], (r[u].y + d.y) * v[u]);
+        r[u] = d;
+      }
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) Xp[(k + u) * ZP] = r[u];
+    }
+    for (; k < L; ++k) {
+      const float2 r = Xp[k * ZP];
+      const float v = Vp[k * ZP];
+      d = make_float2((r.x + d.x) * v, (r.y + d.y) * v);
+      Xp[k * ZP] = d;
+    }
+    // back substitution
+    float2 n = d;
+    k = L - 2;
+    for (; k - (ZB - 1) >= k0; k -= ZB) {
+      float2 r[ZB];
+      float v[ZB];
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) {
+        r[u] = Xp[(k - u) * ZP];
+        v[u] = Vp[(k - u) * ZP];
+      }
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) {
+        n = make_float2(fmaf(v[u], n.x, r[u].x), fmaf(v[u], n.y, r[u].y));
+        r[u] = n;
+      }
+#pragma unroll
+      for (int u = 0; u < ZB; ++u) Xp[(k - u) * ZP] = r[u];
+    }
+    for (; k >= k0; --k) {
+      const float2 r = Xp[k * ZP];
+      const float v = Vp[k * ZP];
+      n = make_float2(fmaf(v, n.x, r.x), fmaf(v, n.y, r.y));
+      Xp[k * ZP] = n;
+    }
+    float2 f = make_float2(0.f, 0.f);
+    if (R.cyclic && !singular) {
+      const float gam = -(lam + 2.f);
+      const float2 y0 = Xp[0], yl = Xp[(L - 1) * ZP];
+      const float q0 = __ldg(qtab + m), ql = __ldg(qtab + (L - 1) * nxy + m);
+      const float den = 1.f + q0 - ql / gam;
+      f = make_float2((y0.x - yl.x / gam) / den, (y0.y - yl.y / gam) / den);
+    }
+    fs[j] = f;
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < ZP * L; idx += blockDim.x) {
-    const int k = idx / ZP, jj = idx - k * ZP;
-    int z = R.z0 + k;
-    if (z >= a.nz) z -= a.nz;
-    if (m0 + jj < nxy) x[(int64_t)z * nxy + m0 + jj] = X[idx];
+  if (ok) {
+    const float2 f = fs[j];
+#pragma unroll 4
+    for (int k = kk; k < L; k += KT) {
+      int z = R.z0 + k;
+      if (z >= a.nz) z -= a.nz;
+      float2 v = X[k * ZP + j];
+      if (R.cyclic) {
+        const float q = __ldg(qtab + k * nxy + m0 + j);
+        v = make_float2(v.x - q * f.x, v.y - q * f.y);
+      }
+      x[z * nxy + m0 + j] = v;
+    }
   }
 }
 
@@ -818,6 +898,8 @@ struct SpectralPlan {
   float2* tw = nullptr;            // twiddles: nx, then ny, then nz values
   float* lam = nullptr;            // eigenvalues: H + 1, then ny, then nz values
   float2* spec = nullptr;          // half spectrum, nz * mxy values
+  float* ztab = nullptr;           // elimination factors of the z solve (k_ztable)
+  float* qtab = nullptr;           // Sherman-Morrison vectors of a cyclic run
   int mxy = 0;
   int lgtp = 0;                    // log2 of the threads per plane
   int ppc = 1;                     // planes per CTA of the plane kernels
@@ -837,6 +919,28 @@ struct SpectralPlan {
   float* hacc = nullptr;           // pinned mirror
 };
 
+namespace {
+SpecArgs args_of(const SpectralPlan* s) {
+  SpecArgs a;
+  a.nx = s->nx;
+  a.ny = s->ny;
+  a.nz = s->nz;
+  a.lgx = s->lgx;
+  a.lgy = s->lgy;
+  a.lgz = s->lgz;
+  a.H = s->nx / 2;
+  a.mxy = s->mxy;
+  a.lgtp = s->lgtp;
+  a.twx = s->tw;
+  a.twy = s->tw + s->nx;
+  a.twz = s->tw + s->nx + s->ny;
+  a.lamx = s->lam;
+  a.lamy = s->lam + s->nx / 2 + 1;
+  a.lamz = a.lamy + s->ny;
+  return a;
+}
+}  // namespace
+
 void spectral_free(lbm_t* h) {
   SpectralPlan* s = h->spec;
   if (!s) return;
@@ -846,6 +950,8 @@ void spectral_free(lbm_t* h) {
   cudaFree(s->tw);
   cudaFree(s->lam);
   cudaFree(s->spec);
+  cudaFree(s->ztab);
+  cudaFree(s->qtab);
   cudaFree(s->r);
   cudaFree(s->psum);
   cudaFree(s->mean_z);
@@ -991,15 +1097,28 @@ lbm_status spectral_setup(lbm_t* h, const uint8_t* solid) {
   }
   int lmax = 0;
   for (const Run& R : runs) lmax = std::max(lmax, R.len);
-  s->zsmem = (size_t)ZP * lmax * (2 + 1 + 1) * sizeof(float);
-  s->runs_fit = s->lgz > 0 || (int)s->zsmem <= optin;
+  s->zsmem = (size_t)ZP * lmax * (2 + 1) * sizeof(float);
+  // the longest run accepted: four words per row and mode
+  s->runs_fit = s->lgz > 0 || (size_t)ZP * lmax * 4 * sizeof(float) <= (size_t)optin;
   if (!s->runs_fit && solid) {
     h->err = "spectral Poisson solver: fluid run along z too long for shared memory";
     return LBM_EINVAL;
   }
   // (without walls yet the plan is provisional: set_walls rebuilds it)
-  if (s->runs_fit && s->lgz < 0 && s->zsmem > 48 * 1024)
-    LBM_CUDA_TRY(h, cudaFuncSetAttribute(k_zsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->zsmem));
+  if (s->runs_fit && s->lgz < 0) {
+    if (s->zsmem > 48 * 1024)
+      LBM_CUDA_TRY(h, cudaFuncSetAttribute(k_zsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->zsmem));
+    const int cyclic = runs[0].cyclic;  // a cyclic run is the only one
+    if (!al((void**)&s->ztab, (size_t)lmax * s->mxy * sizeof(float)) ||
+        (cyclic && !al((void**)&s->qtab, (size_t)lmax * s->mxy * sizeof(float)))) {
+      spectral_free(h);
+      h->err = "spectral Poisson allocation failed";
+      return LBM_ENOMEM;
+    }
+    LBM_CUDA_TRY(h, cudaStreamSynchronize(nullptr));  // the eigenvalues are on the device
+    k_ztable<<<nblk(s->mxy, 128), 128, 0, h->st>>>(s->ztab, s->qtab, lmax, cyclic, args_of(s));
+    LBM_CUDA_TRY(h, cudaGetLastError());
+  }
   h->charge_mean_z = (s->nruns == 1 && s->nplanes == nz) ? s->mean_z : nullptr;
   h->charge_means_ready = false;
   s->plane_smem = (size_t)s->ppc * plane_smem_words(nx, ny) * sizeof(float2);
@@ -1015,26 +1134,6 @@ lbm_status spectral_setup(lbm_t* h, const uint8_t* solid) {
 }
 
 namespace {
-
-SpecArgs args_of(const SpectralPlan* s) {
-  SpecArgs a;
-  a.nx = s->nx;
-  a.ny = s->ny;
-  a.nz = s->nz;
-  a.lgx = s->lgx;
-  a.lgy = s->lgy;
-  a.lgz = s->lgz;
-  a.H = s->nx / 2;
-  a.mxy = s->mxy;
-  a.lgtp = s->lgtp;
-  a.twx = s->tw;
-  a.twy = s->tw + s->nx;
-  a.twz = s->tw + s->nx + s->ny;
-  a.lamx = s->lam;
-  a.lamy = s->lam + s->nx / 2 + 1;
-  a.lamz = a.lamy + s->ny;
-  return a;
-}
 
 // Norm slot i: 2 NACC partial sums (residual^2, then source^2, in
 // fixed-point units squared).
@@ -1135,7 +1234,7 @@ cudaError_t spec_zinv(lbm_t* h) {
     }
   } else {
     dim3 g(nblk(s->mxy, ZP), s->nruns);
-    k_zsolve<<<g, 128, s->zsmem, h->st>>>(s->spec, s->runs, a);
+    k_zsolve<<<g, ZT, s->zsmem, h->st>>>(s->spec, s->runs, s->ztab, s->qtab, a);
   }
   const unsigned gp = (unsigned)((s->nplanes + s->ppc - 1) / s->ppc);
   k_plane_inv<<<gp, s->ppc << s->lgtp, s->plane_smem, h->st>>>(
