@@ -432,6 +432,10 @@ lbm_status spectral_setup(lbm_t* h, const uint8_t* solid_host);
 void spectral_free(lbm_t* h);
 lbm_status spectral_solve(lbm_t* h, double tol, int maxit, int* iters,
                           double* rel_res);
+// Source means of a lattice with wall planes from the charge pass's partial
+// sums over CTAs of ct nodes; false (nothing launched) for one periodic run
+// (charge_mean_z), or when a plane is not a whole number of CTAs.
+bool spectral_run_means(lbm_t* h, int ct);
 // Whole-step graphs: build (if needed) and replay nsteps steps; reads the
 // device status once at the end.
 lbm_status spectral_graph_steps(lbm_t* h, int nsteps);

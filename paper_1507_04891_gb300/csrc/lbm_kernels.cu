@@ -958,13 +958,20 @@ cudaError_t launch_init_species(lbm_t* h, int s, const double* n0,
 }
 
 namespace {
+// CTA size of the charge pass; with wall planes at most a plane (64 nodes or
+// more), so that the partial sums add up to planes (spectral_run_means).
+int charge_cta(const lbm_t* h) {
+  const int nxy = h->cfg.nx * h->cfg.ny;
+  return h->spec && h->has_walls ? std::min(h->charge_threads, nxy) : h->charge_threads;
+}
+
 // The charge pass: the source of the current populations into out (the
 // Poisson source, or the scatter's accumulator), per-CTA partial sums into
 // ps.part; returns the number of partials.
 int charge_pass(lbm_t* h, int64_t* out) {
   // one node per thread (the pulled loads of a node are independent and all
   // in flight); per-CTA partial sums instead of same-address atomics
-  const int ct = h->charge_threads;
+  const int ct = charge_cta(h);
   const int nb = (int)nblocks(h->N, ct);
   const float k = (float)(4.0 * 3.14159265358979323846 * h->cfg.bjerrum);
   // reference part of the source, 4 pi l_B sum_alpha z^alpha n_ref^alpha,
@@ -1073,6 +1080,11 @@ cudaError_t launch_charge(lbm_t* h) {
     h->scat_valid = false;
   } else {
     nbq = charge_pass(h, h->ps.src);
+    // wall planes: the source means of the runs (the total is not used)
+    if (h->has_walls && spectral_run_means(h, charge_cta(h))) {
+      h->charge_means_ready = true;
+      return cudaGetLastError();
+    }
     k_sum_partials<<<1, 1024, 0, h->st>>>(h->ps.part, nbq, h->ps.dsum, h->charge_mean_z,
                                           h->cfg.nz, 1.0 / (double)h->nfluid, h->charge_step);
     ++h->launches;
@@ -1137,6 +1149,7 @@ cudaError_t launch_psi_from_double(lbm_t* h, const double* in, int64_t* psi) {
 }
 
 cudaError_t launch_src_from_rho(lbm_t* h, const double* rho_dev) {
+  h->charge_means_ready = false;  // means of an earlier charge pass no solve followed
   const double k = 4.0 * 3.14159265358979323846 * h->cfg.bjerrum;
   k_src_from_rho<<<(unsigned)std::min<int64_t>(nblocks(h->N, 256), h->grid_cap), 256, 0,
                    h->st>>>(rho_dev, h->links, h->wsrc, h->ps.src, h->ps.dsum, h->ps.label,
