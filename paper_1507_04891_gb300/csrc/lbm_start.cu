@@ -58,55 +58,40 @@ inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 enum { ST_VALID = 0, ST_RING = 1, ST_TERMS = 2, ST_USED = 3 };
 static_assert(ST_RING == START_RING_IDX, "ring position index shared with the charge pass");
 
-// Least-squares coefficients over the first m stored differences:
-// Cholesky of the Gram matrix G (K x K, row-major) with a relative diagonal
-// load of 1e-10 against rounding, rows and columns from m on replaced by the
-// identity so that every loop has the compile-time bound K (the factors stay
-// in registers).  Returns false when a pivot is not positive or a
-// coefficient is not finite.
-__device__ bool solve_gram(const double* __restrict__ G, const double* __restrict__ rhs, int m,
-                           double* c) {
-  double L[K][K];
+// Least-squares coefficients over the first m stored differences, by one
+// warp: Gauss-Jordan elimination in FP64 (the matrix is symmetric positive
+// definite, so no pivoting) of the Gram matrix G (K x K, row-major) with a
+// relative diagonal load of 1e-10 against rounding, rows and columns from m
+// on replaced by the identity.  Lane i K + j holds entry (i, j), lane
+// K K + i the right-hand side of row i.  Returns false in every lane when a
+// pivot is not positive or a coefficient is not finite; else lane K K + i
+// returns coefficient i.
+__device__ bool solve_gram(const double* G, const double* rhs, int m, double& c) {
+  const int lane = threadIdx.x & 31;
+  const bool mat = lane < K * K;
+  const int i = mat ? lane / K : min(lane - K * K, K - 1), j = mat ? lane - i * K : K;
   double load = 0.0;
 #pragma unroll
-  for (int i = 0; i < K; ++i)
-    if (i < m) load += G[i * K + i];
+  for (int q = 0; q < K; ++q)
+    if (q < m) load += G[q * K + q];
   load = 1e-10 * load / m + 1e-300;
+  double v;
+  if (mat) v = (i < m && j < m) ? G[i * K + j] + (i == j ? load : 0.0) : (i == j ? 1.0 : 0.0);
+  else v = i < m ? rhs[i] : 0.0;
   bool ok = true;
 #pragma unroll
-  for (int i = 0; i < K; ++i) {
-#pragma unroll
-    for (int j = 0; j <= i; ++j) {
-      double v;
-      if (i < m && j < m) v = G[i * K + j] + (i == j ? load : 0.0);
-      else v = (i == j) ? 1.0 : 0.0;
-#pragma unroll
-      for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
-      if (i == j) {
-        ok = ok && v > 0.0;
-        L[i][i] = sqrt(v > 0.0 ? v : 1.0);
-      } else {
-        L[i][j] = v / L[j][j];
-      }
-    }
+  for (int k = 0; k < K; ++k) {
+    const double p = __shfl_sync(0xffffffffu, v, k * K + k);
+    ok = ok && p > 0.0;
+    const double f = __shfl_sync(0xffffffffu, v, i * K + k) / (p > 0.0 ? p : 1.0);
+    const double row = __shfl_sync(0xffffffffu, v, mat ? k * K + j : K * K + k);
+    if (i != k) v -= f * row;
   }
-  double y[K];
-#pragma unroll
-  for (int i = 0; i < K; ++i) {
-    double v = i < m ? rhs[i] : 0.0;
-#pragma unroll
-    for (int k = 0; k < i; ++k) v -= L[i][k] * y[k];
-    y[i] = v / L[i][i];
-  }
-#pragma unroll
-  for (int i = K - 1; i >= 0; --i) {
-    double v = y[i];
-#pragma unroll
-    for (int k = i + 1; k < K; ++k) v -= L[k][i] * c[k];
-    c[i] = v / L[i][i];
-    ok = ok && isfinite(c[i]);
-  }
-  return ok;
+  // the diagonal is left: row i's right-hand side over it
+  const double d = __shfl_sync(0xffffffffu, v, i * K + i);
+  c = v / (d != 0.0 ? d : 1.0);
+  ok = ok && (mat || isfinite(c));
+  return __all_sync(0xffffffffu, ok);
 }
 
 // Pass 1 (one cell per thread): D_0 = s(t) - s(t-1) against D_0 and the
@@ -156,26 +141,38 @@ __global__ void __launch_bounds__(DOT_THREADS) k_start_dots(const int64_t* __res
 
 // Pass 2 (one CTA): the inner products g_j = <D_0, D_j> from the partials
 // (compensated FP32 sums in a fixed order), the coefficients over the
-// m = min(K, valid - 1) stored differences (fewer when the factorisation
-// fails; the 5 x 5 factorisation is the only FP64 arithmetic), the Gram
+// m = min(K, valid - 1) stored differences (fewer when the elimination
+// fails; the K x K elimination is the only FP64 arithmetic), the Gram
 // matrix of the next step (D_0 becomes D_1) and the bookkeeping.
-__global__ void __launch_bounds__(256) k_start_solve(const float* __restrict__ part, int nctas,
-                                                     double* __restrict__ gram,
-                                                     float* __restrict__ coef,
-                                                     int* __restrict__ state, int advance) {
+// Latency-bound: the elimination runs in one warp, an entry per lane, where
+// a thread that factorised the matrix alone spent most of the kernel
+// (porous 128^3: 18.4 -> 9.1 us; 32x8x52: 14.3 -> 5.9 us).
+constexpr int SOLVE_THREADS = 512;
+__global__ void __launch_bounds__(SOLVE_THREADS) k_start_solve(const float* __restrict__ part,
+                                                               int nctas, double* __restrict__ gram,
+                                                               float* __restrict__ coef,
+                                                               int* __restrict__ state,
+                                                               int advance) {
+  constexpr int NW = SOLVE_THREADS / 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ float rh[K + 1][NW], rl[K + 1][NW];
+  __shared__ double Gs[K * K], g[K + 1];
+  if (threadIdx.x < K * K) Gs[threadIdx.x] = gram[threadIdx.x];
+  const int valid = state[ST_VALID], r = state[ST_RING];
   float hi[K + 1], lo[K + 1];
 #pragma unroll
   for (int j = 0; j <= K; ++j) hi[j] = lo[j] = 0.f;
-  for (int c0 = threadIdx.x; c0 < nctas; c0 += 8 * blockDim.x) {
-    float x[8][K + 1];
+  constexpr int U = 8;
+  for (int c0 = threadIdx.x; c0 < nctas; c0 += U * SOLVE_THREADS) {
+    float x[U][K + 1];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int c = c0 + u * blockDim.x;
+    for (int u = 0; u < U; ++u) {
+      const int c = c0 + u * SOLVE_THREADS;
 #pragma unroll
       for (int j = 0; j <= K; ++j) x[u][j] = c < nctas ? part[(int64_t)c * (K + 1) + j] : 0.f;
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int j = 0; j <= K; ++j) two_sum_add(hi[j], lo[j], x[u][j]);
   }
@@ -188,56 +185,44 @@ __global__ void __launch_bounds__(256) k_start_solve(const float* __restrict__ p
       two_sum_add(hi[j], lo[j], oh);
       lo[j] += ol;
     }
-  }
-  __shared__ float rh[8][K + 1], rl[8][K + 1];
-  __shared__ double Gs[K * K];
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int j = 0; j <= K; ++j) {
-      rh[threadIdx.x >> 5][j] = hi[j];
-      rl[threadIdx.x >> 5][j] = lo[j];
+    if (lane == 0) {
+      rh[j][wid] = hi[j];
+      rl[j][wid] = lo[j];
     }
-  if (threadIdx.x < K * K) Gs[threadIdx.x] = gram[threadIdx.x];
+  }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  double g[K + 1];
+  if (wid <= K) {  // warp j joins the warps' sums of product j
+    float h = lane < NW ? rh[wid][lane] : 0.f, l = lane < NW ? rl[wid][lane] : 0.f;
 #pragma unroll
-  for (int j = 0; j <= K; ++j) {
-    float h = 0.f, l = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      two_sum_add(h, l, rh[w][j]);
-      l += rl[w][j];
+    for (int off = NW / 2; off > 0; off >>= 1) {
+      const float oh = __shfl_down_sync(0xffffffffu, h, off);
+      const float ol = __shfl_down_sync(0xffffffffu, l, off);
+      two_sum_add(h, l, oh);
+      l += ol;
     }
-    g[j] = (double)h + (double)l;
+    if (lane == 0) g[wid] = (double)h + (double)l;
   }
-  double G[K * K];
-#pragma unroll
-  for (int q = 0; q < K * K; ++q) G[q] = Gs[q];
-  const int valid = state[ST_VALID];
+  __syncthreads();
+  if (wid != 0) return;
   int m = min(K, valid - 1);
-  double c[K];
-#pragma unroll
-  for (int j = 0; j < K; ++j) c[j] = 0.0;
+  double c = 0.0;
   // rhs[j] = <D_0, D_{j+1}> = g[j + 1]; G[i][j] = <D_{i+1}, D_{j+1}>
   for (; m > 0; --m)
-    if (solve_gram(G, g + 1, m, c)) break;
-#pragma unroll
-  for (int j = 0; j < K; ++j) coef[j] = (m > 0 && j < m) ? (float)c[j] : 0.0f;
-  // the next step's Gram matrix: D_0 .. D_{K-2} become D_1 .. D_{K-1}
-#pragma unroll
-  for (int i = 1; i < K; ++i)
-#pragma unroll
-    for (int j = 1; j < K; ++j) gram[i * K + j] = G[(i - 1) * K + (j - 1)];
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    gram[j] = g[j];
-    gram[j * K] = g[j];
+    if (solve_gram(Gs, g + 1, m, c)) break;
+  if (lane >= K * K && lane < K * K + K) {
+    const int j = lane - K * K;
+    coef[j] = (m > 0 && j < m) ? (float)c : 0.0f;
   }
-  const int r = state[ST_RING];
-  state[ST_TERMS] = max(m, 0);
-  if (advance) state[ST_RING] = (r + 1) % K;
-  state[ST_VALID] = min(valid + 1, K + 1);
+  // the next step's Gram matrix: D_0 .. D_{K-2} become D_1 .. D_{K-1}
+  if (lane < K * K) {
+    const int i = lane / K, j = lane - i * K;
+    gram[lane] = i == 0 ? g[j] : (j == 0 ? g[i] : Gs[(i - 1) * K + j - 1]);
+  }
+  if (lane == 0) {
+    state[ST_TERMS] = max(m, 0);
+    if (advance) state[ST_RING] = (r + 1) % K;
+    state[ST_VALID] = min(valid + 1, K + 1);
+  }
 }
 
 // Pass 3: psi(t-1) + sum_j c_j P_j with P_1 = psi(t-1) - psi(t-2) (fresh)
@@ -581,7 +566,7 @@ cudaError_t start_fit(lbm_t* h, cudaStream_t st, bool last) {
                                                  H.part);
     ++h->launches;
   }
-  k_start_solve<<<1, 256, 0, st>>>(H.part, nparts, H.gram, H.coef, H.state, last ? 1 : 0);
+  k_start_solve<<<1, SOLVE_THREADS, 0, st>>>(H.part, nparts, H.gram, H.coef, H.state, last ? 1 : 0);
   ++h->launches;
   return cudaGetLastError();
 }
