@@ -20,18 +20,20 @@ BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "liblbm_gb300.so")
 # (source, object name, extra nvcc flags): the stream/collide unit is compiled
 # once per population storage format (LBM_FP32 = 0, LBM_FP16_SHIFT = 1,
-# LBM_BF16_SHIFT = 2) so that its many kernel instances build in parallel
+# LBM_BF16_SHIFT = 2) and number of nodes per thread so that its many kernel
+# instances build in parallel
 UNITS = [("lbm_api.cu", "lbm_api", []), ("lbm_kernels.cu", "lbm_kernels", []),
-         ("lbm_collide.cu", "lbm_collide_fp32", ["-DLBM_COLLIDE_STORAGE=0"]),
-         ("lbm_collide.cu", "lbm_collide_fp16", ["-DLBM_COLLIDE_STORAGE=1"]),
-         ("lbm_collide.cu", "lbm_collide_bf16", ["-DLBM_COLLIDE_STORAGE=2"]),
+         *[("lbm_collide.cu", "lbm_collide_%s_%d" % (fmt, nv),
+            ["-DLBM_COLLIDE_STORAGE=%d" % st, "-DLBM_COLLIDE_NODES=%d" % nv])
+           for st, fmt, nv in ((0, "fp32", 1), (1, "fp16", 1), (1, "fp16", 2), (2, "bf16", 1),
+                               (2, "bf16", 2))],
          ("lbm_poisson.cu", "lbm_poisson", []), ("lbm_spectral.cu", "lbm_spectral", []),
          ("lbm_start.cu", "lbm_start", []), ("lbm_nn.cu", "lbm_nn", []),
          ("lbm_noalloc.cu", "lbm_noalloc", [])]
 SOURCES = sorted({u[0] for u in UNITS})
 HEADERS = ["lbm_internal.cuh", "lbm_lattice.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-split-compile=4", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "-I", os.path.join(ROOT, "include")]
 
 

@@ -345,7 +345,9 @@ void lbm_destroy(lbm_t* h) {
   cudaFree(h->scat_acc);
   cudaFree(h->scat_tot);
   cudaFree(h->links);
+  cudaFree(h->wcls);
   cudaFree(h->wallq);
+  cudaFree(h->wallg);
   cudaFree(h->wsrc);
   cudaFree(h->dred);
   if (h->hrec) cudaFreeHost(h->hrec);
@@ -423,6 +425,7 @@ lbm_status lbm_set_walls(lbm_t* h, const uint8_t* solid, const double* sigma) {
   if (cudaMalloc(&sc.p, N) != cudaSuccess) return fail(h, LBM_ENOMEM, "scratch allocation failed");
   lbm_status s = LBM_OK;
   if (!h->links) s = dev_alloc(h, &h->links, N);
+  if (s == LBM_OK && !h->wcls) s = dev_alloc(h, &h->wcls, (size_t)((N + 31) / 32));
   if (s != LBM_OK) return s;
   LBM_CUDA_TRY(h, cudaMemcpy(sc.p, solid, N, cudaMemcpyHostToDevice));
   h->has_walls = true;
@@ -437,10 +440,17 @@ lbm_status lbm_set_walls(lbm_t* h, const uint8_t* solid, const double* sigma) {
     for (int64_t i = 0; i < N; ++i) wfx[i] = llrint(k4 * wd[i] * PSI_SCALE);
     LBM_CUDA_TRY(h, cudaMemcpy(h->wallq, q.data(), N * sizeof(float), cudaMemcpyHostToDevice));
     LBM_CUDA_TRY(h, cudaMemcpy(h->wsrc, wfx.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice));
+    if (h->cfg.bjerrum > 0.0) {
+      if (!h->wallg && (s = dev_alloc(h, &h->wallg, 3 * (size_t)N)) != LBM_OK) return s;
+      LBM_CUDA_TRY(h, cudaStreamSynchronize(nullptr));  // the charges are on the device
+      LBM_CUDA_TRY(h, launch_wall_gradient(h));
+    }
   } else {
     cudaFree(h->wallq);
+    cudaFree(h->wallg);
     cudaFree(h->wsrc);
     h->wallq = nullptr;
+    h->wallg = nullptr;
     h->wsrc = nullptr;
   }
   h->nfluid = nfluid;

@@ -1,19 +1,20 @@
-// The fused stream/collide kernel of one population storage format.  This
-// file is compiled once per format (LBM_COLLIDE_STORAGE = LBM_FP32,
-// LBM_FP16_SHIFT, LBM_BF16_SHIFT), so that the instances of the kernel (species
-// count, walls, charge, diagnostics) build in parallel; each object defines
-// collide_dispatch<LBM_COLLIDE_STORAGE>.
+// The fused stream/collide kernel of one population storage format and
+// number of nodes per thread.  This file is compiled once per format
+// (LBM_COLLIDE_STORAGE = LBM_FP32, LBM_FP16_SHIFT, LBM_BF16_SHIFT) and nodes
+// per thread (LBM_COLLIDE_NODES = 1, 2), so that the instances of the kernel
+// (species count, walls, charge, diagnostics) build in parallel; each object
+// defines collide_dispatch<LBM_COLLIDE_STORAGE, LBM_COLLIDE_NODES>.
 #include "lbm_lattice.cuh"
 
-#ifndef LBM_COLLIDE_STORAGE
-#error "compile with -DLBM_COLLIDE_STORAGE=<storage code>"
+#if !defined(LBM_COLLIDE_STORAGE) || !defined(LBM_COLLIDE_NODES)
+#error "compile with -DLBM_COLLIDE_STORAGE=<storage code> -DLBM_COLLIDE_NODES=<1 or 2>"
 #endif
 
 namespace lbm_gb300 {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Fused stream + collide, one thread per node, all S species in registers.
+// Fused stream + collide, all S species of a thread's nodes in registers.
 //   1. pull the 19*S populations f_p^alpha(r, t), as deviations from
 //      w_p n_ref                                            (Eq. latboeq, lhs)
 //   2. n^alpha, bare u^alpha = sum c f / n, barycentric u   (Sec. 3 definitions)
@@ -35,6 +36,18 @@ namespace {
 //      and a count of nodes whose density entering the step was not finite
 //      and positive, written to a[blockIdx.x * DIAG_NQ + k].
 // ---------------------------------------------------------------------------
+// NV nodes per thread (V<NV>, lbm_lattice.cuh): one in FP32, two consecutive
+// x nodes in the 16-bit formats when nx is even.  The 16-bit kernel is bound
+// by instruction issue and by the latency between its instructions, not by
+// HBM: with two nodes the arithmetic issues packed FP32 instructions, the
+// populations wait in registers as packed pairs, addresses are formed once
+// per pair and directions without an x component move as one word
+// (ternary 128^3, FP16: 1.10e8 -> 6.4e7 warp instructions, 122.7 -> 101.7 us
+// in ncu; 64 slits of 32x32 342 -> 271 us in the step).  In FP32 two nodes
+// per thread need over 200 registers: 8 warps per SM instead of 16, 234 us
+// against 180, and a form that landed the next tile in shared memory behind
+// the arithmetic 223 us, so FP32 keeps one node.
+//
 // Charge scatter: the target of a stored population h*_p(r) is r + c_p
 // (it is pulled there at the next step).  Targets are grouped by their row
 // offset (dy, dz) = (c_y, c_z), nine groups; GRP numbers them.  Five groups
@@ -46,14 +59,39 @@ __host__ __device__ __forceinline__ constexpr int XGRP_OF(int dy, int dz) {
   return dz == 0 ? (dy == 0 ? 0 : (dy == 1 ? 1 : 2)) : (dz == 1 ? 3 : 4);
 }
 __host__ __device__ __forceinline__ constexpr int XGRP(int p) { return XGRP_OF(CY(p), CZ(p)); }
+// group of XGRP j
+__host__ __device__ __forceinline__ constexpr int GRP_OF_X(int j) {
+  return j == 0 ? 4 : (j == 1 ? 5 : (j == 2 ? 3 : (j == 3 ? 7 : 1)));
+}
 
-// (p is a constant once the direction loops are unrolled, so the sums stay
-// in registers)
-__device__ __forceinline__ void scat_add(int p, float (&q0)[9], float (&qp)[5], float (&qm)[5],
-                                         float v) {
-  if (CX(p) == 0) q0[GRP(p)] += v;
-  else if (CX(p) == 1) qp[XGRP(p)] += v;
-  else qm[XGRP(p)] += v;
+struct Scat {
+  float q0[9], qp[5], qm[5];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int g = 0; g < 9; ++g) q0[g] = 0.f;
+#pragma unroll
+    for (int g = 0; g < 5; ++g) qp[g] = qm[g] = 0.f;
+  }
+  // (p is a constant once the direction loops are unrolled, so the sums stay
+  // in registers)
+  __device__ __forceinline__ void add(int p, float kw, float h) {
+    float& q = CX(p) == 0 ? q0[GRP(p)] : (CX(p) == 1 ? qp[XGRP(p)] : qm[XGRP(p)]);
+    q = fmaf(kw, h, q);
+  }
+};
+
+// Nearest fixed-point integer of a float below 2^62: the part above 2^32
+// (rounded, so that the rest is exact in FP32 and signed) and the rest, each
+// by the 32-bit conversion (a rest of exactly 2^31 loses one unit of 2^-52).
+// Seven instructions; f32_to_i64_rn's shifts of 64-bit words took about
+// three times as many, and the scatter converts 9 to 14 sums per node.
+// With the 32-bit node offsets and the reciprocal of vrcp the kernel with the
+// scatter went from 1.30e8 to 1.06e8 warp instructions at 128^3, 178.6 ->
+// 155.0 us in ncu, 180 -> 166 in the step.
+__device__ __forceinline__ unsigned long long scat_fixed(float c) {
+  const int hi = __float2int_rn(c * 2.3283064365386963e-10f);
+  const int lo = __float2int_rn(fmaf(-4294967296.0f, (float)hi, c));
+  return (unsigned long long)(((long long)hi << 32) + (long long)lo);
 }
 
 // A warp holds 32 consecutive nodes of one x row (nx is a multiple of 32).
@@ -67,19 +105,16 @@ __device__ __forceinline__ void scat_add(int p, float (&q0)[9], float (&qp)[5], 
 // FP32 sums are formed in a fixed order, so every run gives the same
 // source).  The node's own target also receives the reference part of the
 // source, once per node.  (x, y, z): the lane's node.
-__device__ __forceinline__ void scatter_charge(const StepArgs& a, int x, int y, int z,
-                                               float (&c0)[9], const float (&cp)[5],
-                                               const float (&cm)[5]) {
+__device__ __forceinline__ void scatter_charge(const StepArgs& a, int x, int y, int z, Scat& c) {
   const int lane = threadIdx.x & 31;
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const bool one = nx == 32;  // the row is this warp: the shuffles wrap it
 #pragma unroll
   for (int j = 0; j < 5; ++j) {
-    const float fl = __shfl_sync(0xffffffffu, cp[j], (lane + 31) & 31);  // lane - 1 sends to x
-    const float fr = __shfl_sync(0xffffffffu, cm[j], (lane + 1) & 31);   // lane + 1 sends to x
-    const int g = j == 0 ? 4 : (j == 1 ? 5 : (j == 2 ? 3 : (j == 3 ? 7 : 1)));  // GRP of XGRP j
-    if (one || lane != 0) c0[g] += fl;
-    if (one || lane != 31) c0[g] += fr;
+    const float fl = __shfl_sync(0xffffffffu, c.qp[j], (lane + 31) & 31);  // lane - 1 sends to x
+    const float fr = __shfl_sync(0xffffffffu, c.qm[j], (lane + 1) & 31);   // lane + 1 sends to x
+    if (one || lane != 0) c.q0[GRP_OF_X(j)] += fl;
+    if (one || lane != 31) c.q0[GRP_OF_X(j)] += fr;
   }
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(a.scat_acc);
   const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
@@ -89,291 +124,534 @@ __device__ __forceinline__ void scatter_charge(const StepArgs& a, int x, int y, 
   const int rowy[3] = {ym * nx, y * nx, yp * nx};
 #pragma unroll
   for (int g = 0; g < 9; ++g) {
-    long long q = (long long)f32_to_i64_rn(c0[g]);
-    if (g == 4) q += a.src_ref;
-    atomicAdd(acc + rowz[g / 3] + rowy[g % 3] + x, (unsigned long long)q);
+    unsigned long long q = scat_fixed(c.q0[g]);
+    if (g == 4) q += (unsigned long long)a.src_ref;
+    atomicAdd(acc + rowz[g / 3] + rowy[g % 3] + x, q);
   }
   if (!one && (lane == 0 || lane == 31)) {
     // the contributions that cross into the neighbouring warp of the row
     const int xt = lane == 0 ? (x == 0 ? nx - 1 : x - 1) : (x == nx - 1 ? 0 : x + 1);
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      const int g = j == 0 ? 4 : (j == 1 ? 5 : (j == 2 ? 3 : (j == 3 ? 7 : 1)));
-      const float v = lane == 0 ? cm[j] : cp[j];
-      atomicAdd(acc + rowz[g / 3] + rowy[g % 3] + xt, (unsigned long long)(long long)f32_to_i64_rn(v));
+    for (int j = 0; j < 5; ++j)
+      atomicAdd(acc + rowz[GRP_OF_X(j) / 3] + rowy[GRP_OF_X(j) % 3] + xt,
+                scat_fixed(lane == 0 ? c.qm[j] : c.qp[j]));
+  }
+}
+
+// c . v for the direction p (a constant once unrolled): additions only.
+template <int NV>
+__device__ __forceinline__ V<NV> cdot(int p, const V<NV>& x, const V<NV>& y, const V<NV>& z) {
+  const int c[3] = {CX(p), CY(p), CZ(p)};
+  const V<NV>* v[3] = {&x, &y, &z};
+  V<NV> r;
+  bool first = true;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (c[d] == 0) continue;
+    // every odd p has its first non-zero component positive or its pair has
+    if (first) r = c[d] > 0 ? *v[d] : V<NV>(0.f) - *v[d];
+    else r = c[d] > 0 ? r + *v[d] : r - *v[d];
+    first = false;
+  }
+  return r;
+}
+
+// Deviation sums of the state after the step over a thread's nodes.
+template <int S>
+struct Sums {
+  float m[S], jx, jy, jz, bad;
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int s = 0; s < S; ++s) m[s] = 0.f;
+    jx = jy = jz = bad = 0.f;
+  }
+};
+
+// The pulled populations of a thread as they came from memory: floats, or
+// for two nodes of a 16-bit format the packed pair (half the registers of
+// the unpacked ones; unpacked where it is used, once for the moments and
+// once for the update).
+template <int ST, int NV>
+struct Raw {
+  V<NV> v;
+  __device__ __forceinline__ V<NV> get() const { return v; }
+  __device__ __forceinline__ void clear(int k) { v.set(k, 0.f); }
+};
+template <>
+struct Raw<LBM_FP16_SHIFT, 2> {
+  uint32_t v;
+  __device__ __forceinline__ V<2> get() const { return Fmt<LBM_FP16_SHIFT>::unpack(v); }
+  __device__ __forceinline__ void clear(int k) { v &= k ? 0x0000ffffu : 0xffff0000u; }
+};
+template <>
+struct Raw<LBM_BF16_SHIFT, 2> {
+  uint32_t v;
+  __device__ __forceinline__ V<2> get() const { return Fmt<LBM_BF16_SHIFT>::unpack(v); }
+  __device__ __forceinline__ void clear(int k) { v &= k ? 0x0000ffffu : 0xffff0000u; }
+};
+
+// Population (s, p): the base address is the same for the whole warp, the
+// node's byte offset one 32-bit number (a plane of 2^30 nodes is at most
+// 2^32 bytes).
+template <class T>
+__device__ __forceinline__ const T* pop_at(const void* base, int64_t plane, uint32_t off) {
+  return reinterpret_cast<const T*>(static_cast<const char*>(base) + plane * (int64_t)sizeof(T) + off);
+}
+
+// Gradient of psi along one axis at a node: mean of the two face gradients,
+// half the difference of the two neighbours between open faces (an exact
+// integer difference, rounded once).  At a wall face the node's own value
+// takes the neighbour's place and the Neumann value of the surface-charge
+// condition is in the wall part w (k_wall_gradient).
+template <bool WALLS>
+__device__ __forceinline__ float axis_gradient(int64_t c, int64_t m, int64_t p, uint32_t wm, uint32_t wp,
+                                               float w) {
+  if (WALLS) {
+    p = wp ? c : p;
+    m = wm ? c : m;
+    return fmaf((float)(p - m), 0.5f * PSI_INV_SCALE_F, w);
+  }
+  return (float)(p - m) * (0.5f * PSI_INV_SCALE_F);
+}
+
+// Potential of NV consecutive nodes.
+template <int NV>
+__device__ __forceinline__ void ld_psi(const int64_t* __restrict__ p, int64_t (&v)[NV]) {
+  if constexpr (NV == 1) {
+    v[0] = *p;
+  } else {
+    const longlong2 w = *reinterpret_cast<const longlong2*>(p);
+    v[0] = w.x;
+    v[1] = w.y;
+  }
+}
+
+// (link: a node of the warp has a wall node beside it)
+template <int NV, bool WALLS>
+__device__ __forceinline__ void psi_gradient_v(const StepArgs& a, uint32_t i, const Nbr& o,
+                                               const uint32_t (&lk)[NV], bool link, V<NV>& gx,
+                                               V<NV>& gy, V<NV>& gz) {
+  const int64_t* __restrict__ ps = a.psi + i;
+  int64_t c[NV] = {}, yp[NV], ym[NV], zp[NV], zm[NV];
+  if (WALLS || NV == 2) ld_psi<NV>(ps, c);
+  ld_psi<NV>(ps + o.dyp, yp);
+  ld_psi<NV>(ps + o.dym, ym);
+  ld_psi<NV>(ps + o.dzp, zp);
+  ld_psi<NV>(ps + o.dzm, zm);
+  const int64_t xl = ps[o.dxm], xr = ps[NV - 1 + o.dxp];
+  V<NV> w[3] = {0.f, 0.f, 0.f};
+  if (WALLS && link && a.wallg) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int k = 0; k < NV; ++k) w[d].set(k, a.wallg[(int64_t)d * a.N + i + k]);
+  }
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    // bit 2: r + x is a wall node; bit 1: r - x; 4: +y; 3: -y; 6: +z; 5: -z
+    const uint32_t l = lk[k];
+    const int64_t m = k == 0 ? xl : c[0], p = k == NV - 1 ? xr : c[NV - 1];
+    gx.set(k, axis_gradient<WALLS>(c[k], m, p, l & 2u, l & 4u, w[0].get(k)));
+    gy.set(k, axis_gradient<WALLS>(c[k], ym[k], yp[k], l & 8u, l & 16u, w[1].get(k)));
+    gz.set(k, axis_gradient<WALLS>(c[k], zm[k], zp[k], l & 32u, l & 64u, w[2].get(k)));
+  }
+}
+
+// The collision of a thread's NV nodes from i on (plane z) and the stores:
+// f the pulled h_p, (gx, gy, gz) the potential's gradient, lk the link words
+// and act the fluid flags of the nodes.
+template <int S, int NV, bool WALLS, bool CHARGED, int ST, bool DIAG, bool PAIR, bool SCAT>
+__device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int z,
+                                              const uint32_t (&lk)[NV], const bool (&act)[NV],
+                                              const Raw<ST, NV> (&f)[S][Q], const V<NV>& gx,
+                                              const V<NV>& gy, const V<NV>& gz, Scat& sc,
+                                              Sums<S>& q) {
+  using T = typename Fmt<ST>::T;
+  using F = V<NV>;
+  T* __restrict__ fout = static_cast<T*>(a.fout) + i;
+  const int64_t N = a.N;
+  // n = n_ref (1 + sum w h), j = n_ref sum c w h  (sum w = 1, sum w c = 0),
+  // summed per weight class (faces p = 1..6, edges 7..18) so that each
+  // population costs additions only
+  F mh[S], n[S], jx[S], jy[S], jz[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    F h[Q];
+#pragma unroll
+    for (int p = 0; p < Q; ++p) h[p] = f[s][p].get();
+    const F sf = ((h[1] + h[2]) + (h[3] + h[4])) + (h[5] + h[6]);
+    F se = h[7];
+#pragma unroll
+    for (int p = 8; p < Q; ++p) se = se + h[p];
+    // x: faces 1 - 2, edges 7 - 8 + 9 - 10 + 11 - 12 + 13 - 14, and so on
+    const F xe = ((h[7] - h[8]) + (h[9] - h[10])) + ((h[11] - h[12]) + (h[13] - h[14]));
+    const F ye = ((h[7] - h[8]) - (h[9] - h[10])) + ((h[15] - h[16]) + (h[17] - h[18]));
+    const F ze = ((h[11] - h[12]) - (h[13] - h[14])) + ((h[15] - h[16]) - (h[17] - h[18]));
+    mh[s] = vfma(F(WT(0)), h[0], vfma(F(WT(1)), sf, F(WT(7)) * se));
+    const float r = a.nref[s];
+    n[s] = vfma(F(r), mh[s], F(r));
+    jx[s] = F(r) * vfma(F(WT(1)), h[1] - h[2], F(WT(7)) * xe);
+    jy[s] = F(r) * vfma(F(WT(1)), h[3] - h[4], F(WT(7)) * ye);
+    jz[s] = F(r) * vfma(F(WT(1)), h[5] - h[6], F(WT(7)) * ze);
+    if (DIAG) {
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+        if (act[k] && (!(n[s].get(k) > 0.f) || !isfinite(n[s].get(k)))) q.bad += 1.f;
+    }
+  }
+
+  F ntot = n[0], Jx = jx[0], Jy = jy[0], Jz = jz[0];
+#pragma unroll
+  for (int s = 1; s < S; ++s) {
+    ntot = ntot + n[s];
+    Jx = Jx + jx[s];
+    Jy = Jy + jy[s];
+    Jz = Jz + jz[s];
+  }
+  const F inv_ntot = vrcp(ntot);
+  // barycentric velocity (equal masses: mass-weighted = number-weighted)
+  const F ux = Jx * inv_ntot, uy = Jy * inv_ntot, uz = Jz * inv_ntot;
+
+  // field: applied minus c_s^2 grad psi
+  F Ex(a.eext[0]), Ey(a.eext[1]), Ez(a.eext[2]);
+  if (CHARGED) {
+    Ex = vfma(F(-CS2), gx, Ex);
+    Ey = vfma(F(-CS2), gy, Ey);
+    Ez = vfma(F(-CS2), gz, Ez);
+  }
+
+  // number-weighted mean of the drag velocities u^a + F_el^a / 2
+  F zn = F(a.valence[0]) * n[0];
+#pragma unroll
+  for (int s = 1; s < S; ++s) zn = vfma(F(a.valence[s]), n[s], zn);
+  const F hzn = F(0.5f) * zn;
+  const F vbx = vfma(hzn, Ex, Jx) * inv_ntot;
+  const F vby = vfma(hzn, Ey, Jy) * inv_ntot;
+  const F vbz = vfma(hzn, Ez, Jz) * inv_ntot;
+  // pair frequencies: the fractions x_b and x_b v_b of every species
+  F px[PAIR ? S : 1], pxv[PAIR ? S : 1][3];
+  if (PAIR) {
+#pragma unroll
+    for (int b = 0; b < S; ++b) {
+      px[b] = n[b] * inv_ntot;
+      const F hz = F(0.5f * a.valence[b]) * n[b];
+      pxv[b][0] = vfma(hz, Ex, jx[b]) * inv_ntot;
+      pxv[b][1] = vfma(hz, Ey, jy[b]) * inv_ntot;
+      pxv[b][2] = vfma(hz, Ez, jz[b]) * inv_ntot;
+    }
+  }
+
+  const float om = a.omega_visc;
+  const float omd = a.omega_drag_z ? a.omega_drag_z[z] : a.omega_drag;
+  uint32_t rnd[NV];
+  if (ST != LBM_FP32) {
+    const uint32_t st = mix32(a.step_dev ? *a.step_dev : a.step);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) rnd[k] = mix32((i + k) * 0x9E3779B9u ^ st);
+  }
+  auto next = [&](int k) -> uint32_t { return ST != LBM_FP32 ? lcg_next(rnd[k]) : 0u; };
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const F inv_n = vrcp(n[s]);
+    const F usx = jx[s] * inv_n, usy = jy[s] * inv_n, usz = jz[s] * inv_n;
+    // force per unit mass (Sec. 2): the electric acceleration and the drag
+    // on the velocities shifted by half of it
+    const F zs(a.valence[s]);
+    F Fx, Fy, Fz;
+    {
+      const F ex = zs * Ex, ey = zs * Ey, ez = zs * Ez, half(0.5f);
+      const F vx = vfma(half, ex, usx), vy = vfma(half, ey, usy), vz = vfma(half, ez, usz);
+      if (PAIR) {
+        // F_drag^a = -(W v_a - M), W = sum_b omega^{ab} x_b,
+        // M = sum_b omega^{ab} x_b v_b (omega^{aa} = 0)
+        F W(0.f), Mx(0.f), My(0.f), Mz(0.f);
+#pragma unroll
+        for (int b = 0; b < S; ++b) {
+          const F w(a.pair[s][b]);
+          W = vfma(w, px[b], W);
+          Mx = vfma(w, pxv[b][0], Mx);
+          My = vfma(w, pxv[b][1], My);
+          Mz = vfma(w, pxv[b][2], Mz);
+        }
+        Fx = ex + (Mx - W * vx);
+        Fy = ey + (My - W * vy);
+        Fz = ez + (Mz - W * vz);
+      } else {
+        Fx = vfma(F(omd), vbx - vx, ex);
+        Fy = vfma(F(omd), vby - vy, ey);
+        Fz = vfma(F(omd), vbz - vz, ez);
+      }
+    }
+    const F usq = vfma(usx, usx, vfma(usy, usy, usz * usz));
+    const F Fu = vfma(Fx, ux, vfma(Fy, uy, Fz * uz));
+    // In deviations, d*_p = (1 - omega) d_p + [omega phi_p + g_p - omega w_p n_ref]
+    // with, per weight w_p,
+    //   omega phi_p + g_p - omega w_p n_ref
+    //     = w_p [omega dn + n (-1.5 omega |u^a|^2 - 3 F.u
+    //                          + 4.5 omega a^2 + 9 (F.c)(u.c))]      (even in c)
+    //     + w_p n 3 (omega a + F.c)                                 (odd in c)
+    // a = u^a.c (phi_perp in its reduced form, the Appendix expression;
+    // g_p of Eq. ourforc).  Divided by w_p n_ref this updates the stored
+    // h = d / (w_p n_ref) directly: h*_p = (1 - omega) h_p + (even' +/- odd') / n_ref,
+    // with the bracket values even', odd' free of w_p.  Every term is of
+    // the size of the deviations.
+    const float inr = 1.0f / a.nref[s];
+    // the per-species factors of the bracket values, once per species:
+    // even' = Ce + Ae a^2 + Be (F.c)(u.c), odd' = Do (omega a + F.c)
+    const F nin = n[s] * F(inr);
+    const F Ae = nin * F(4.5f * om), Be = nin * F(9.0f), Do = nin * F(3.0f);
+    const F Ce = vfma(nin, vfma(F(-1.5f * om), usq, F(-3.0f) * Fu), F(om) * mh[s]);
+    const F om_(om);
+    // moving populations first; the rest population then takes
+    // d*_0 = dn - sum_{p>0} d*_p over the stored (rounded) moving values,
+    // i.e. h*_0 = (sum w h - sum_{p>0} w h*_p) / w_0, which holds exactly
+    // in real arithmetic (phi_perp carries mass n, g_p none) and keeps the
+    // rounding of the weights and of 16-bit stores from drifting the
+    // species mass.
+    // Directions come in opposite pairs (p, p+1), c_{p+1} = -c_p: a = u^a.c,
+    // F.c and u.c flip sign, so each pair shares the even part and takes
+    // +/- the odd part.
+    const F omm(1.0f - om);
+    F mvf(0.f), mve(0.f);  // stored values summed, faces and edges
+    float mjx = 0.f, mjy = 0.f, mjz = 0.f;
+#pragma unroll
+    for (int p = 1; p < Q; p += 2) {
+      const F av = cdot<NV>(p, usx, usy, usz);
+      const F fc = cdot<NV>(p, Fx, Fy, Fz);
+      const F uc = cdot<NV>(p, ux, uy, uz);
+      const F even = vfma(Ae * av, av, vfma(Be * fc, uc, Ce));
+      const F odd = Do * vfma(om_, av, fc);
+      F ha = vfma(omm, f[s][p].get(), even + odd), hb = vfma(omm, f[s][p + 1].get(), even - odd);
+      T* pa = fout + (int64_t)(s * Q + p) * N;
+      if constexpr (NV == 2) {
+        Fmt<ST>::sth_sr22(pa, ha.a, pa + N, hb.a, next(0), next(1));
+      } else {
+        const float2 hs = Fmt<ST>::sth_sr2(pa, ha.a, pa + N, hb.a, next(0));
+        ha = hs.x;
+        hb = hs.y;
+      }
+      const F pr = ha + hb;  // same weight for p and p + 1
+      if (p <= 6) mvf = mvf + pr;
+      else mve = mve + pr;
+      if constexpr (SCAT) {
+        // charge these stored values carry to r + c_p and r - c_p
+        // (zero for a neutral species)
+        const float kw = a.scat_k[s] * WT(p);
+        sc.add(p, kw, ha.a);
+        sc.add(p + 1, kw, hb.a);
+      }
+      // momentum carried by the pair at the next step: h*_p moves along
+      // c_p unless r + c_p is a wall node (bit p+1), then it is pulled
+      // back along -c_p; h*_{p+1} likewise with bit p
+      if (DIAG) {
+        float mj = 0.f;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          if (WALLS) {
+            if (act[k])
+              mj += (((lk[k] >> (p + 1)) & 1u) ? -ha.get(k) : ha.get(k)) -
+                    (((lk[k] >> p) & 1u) ? -hb.get(k) : hb.get(k));
+          } else {
+            mj += ha.get(k) - hb.get(k);
+          }
+        }
+        if (CX(p)) mjx += CX(p) * WT(p) * mj;
+        if (CY(p)) mjy += CY(p) * WT(p) * mj;
+        if (CZ(p)) mjz += CZ(p) * WT(p) * mj;
+      }
+    }
+    const F moved = vfma(F(WT(1)), mvf, F(WT(7)) * mve);
+    F h0 = (mh[s] - moved) * F(INV_WT(0));
+    T* p0 = fout + (int64_t)(s * Q) * N;
+    if constexpr (NV == 2) Fmt<ST>::sth_sr_pair(p0, h0.a, next(0), next(1));
+    else h0 = Fmt<ST>::sth_sr(p0, h0.a, next(0));
+    if constexpr (SCAT) sc.add(0, a.scat_k[s] * WT(0), h0.a);
+    if (DIAG) {
+      const float r = a.nref[s];
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+        if (act[k]) q.m[s] += r * fmaf(WT(0), h0.get(k), moved.get(k));
+      q.jx += r * mjx;
+      q.jy += r * mjy;
+      q.jz += r * mjz;
     }
   }
 }
 
-// Registers: up to 128 per thread (two 256-thread CTAs per SM), 255 for four
-// species.  The 16-bit ternary kernel without walls is capped at 96: it is
-// bound by instruction issue, and 20 warps per SM (128-thread CTAs) instead
-// of 16 issue more often than the few spilled registers cost (measured at
-// 128^3: 133 -> 127 us per launch; 88 registers: 130 us).
-template <int S, bool WALLS, int ST>
-constexpr int collide_maxnreg() {
-  return S >= 4 ? 255 : ((ST != LBM_FP32 && !WALLS && S == 3) ? 96 : 128);
+// The diagnostics sums of a thread as the DIAG_NQ quantities of the partials.
+template <int S>
+__device__ __forceinline__ void diag_quantities(const StepArgs& a, const Sums<S>& q,
+                                                float (&v)[DIAG_NQ]) {
+#pragma unroll
+  for (int k = 0; k < DIAG_NQ; ++k) v[k] = 0.f;
+  float qc = 0.f;
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    v[s] = q.m[s];
+    qc += a.valence[s] * q.m[s];
+  }
+  v[MAX_SPECIES + 0] = q.jx;
+  v[MAX_SPECIES + 1] = q.jy;
+  v[MAX_SPECIES + 2] = q.jz;
+  v[MAX_SPECIES + 3] = qc;
+  v[MAX_SPECIES + 4] = q.bad;
 }
 
-template <int S, bool WALLS, bool CHARGED, int ST, bool DIAG, bool PAIR, bool SCAT>
-__global__ void __launch_bounds__(256) __maxnreg__((collide_maxnreg<S, WALLS, ST>()))
+// Registers: up to 128 per thread (16 warps per SM), 255 for four species.
+// Two nodes per thread of three species: 168 (12 warps); ternary 128^3 FP16
+// took 110 us with 168 in ncu, 123 with 128 (spills), 108 against 102 with
+// 144; 64 slits 271 us with 168, 331 with 200, 322 with 255.
+template <int S, int NV>
+constexpr int collide_maxnreg() {
+  return S >= 4 ? 255 : (S == 3 && NV == 2 ? 168 : 128);
+}
+
+template <int S, int NV, bool WALLS, bool CHARGED, int ST, bool DIAG, bool PAIR, bool SCAT>
+__global__ void __launch_bounds__(256) __maxnreg__((collide_maxnreg<S, NV>()))
     k_stream_collide(const StepArgs a) {
   using T = typename Fmt<ST>::T;
   // a speculative launch the step has decided against (same for every
   // thread of the grid)
   if (a.skip && *a.skip) return;
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  // deviation sums of the state after the step: masses, momentum, charge
-  float qm[S], qjx = 0.f, qjy = 0.f, qjz = 0.f, qbad = 0.f;
-#pragma unroll
-  for (int s = 0; s < S; ++s) qm[s] = 0.f;
-  // (SCAT) charge sent to the next step's source, per target group
-  float c0[9], cp[5], cm[5];
-#pragma unroll
-  for (int g = 0; g < 9; ++g) c0[g] = 0.f;
-#pragma unroll
-  for (int g = 0; g < 5; ++g) cp[g] = cm[g] = 0.f;
-  uint32_t lk = 0;
+  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) * NV;
+  Sums<S> q;
+  q.clear();
+  Scat sc;  // (SCAT) charge sent to the next step's source
+  if constexpr (SCAT) sc.clear();
   const bool inrange = i < (uint32_t)a.N;
-  bool active = inrange;
-  if (WALLS && inrange) {
-    lk = a.links[i];
-    active = !(lk & LINK_SOLID);
+  uint32_t lk[NV];
+  bool act[NV], work = inrange, mixed = false;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) lk[k] = 0u;
+  if (WALLS) {
+    // The class of the warp's nodes (a byte per 32 nodes, from the caches)
+    // tells whether the link words matter: warps without wall nodes or wall
+    // neighbours pull at once, warps of wall nodes only do nothing, and only
+    // the others wait for their link words, which choose the addresses of
+    // the pulls.  Wall nodes in a warp with fluid nodes run the same
+    // instructions and store what they computed from zeros into their own
+    // slots (which no pull reads): every store of the warp then covers whole
+    // sectors, so the L2 need not fetch the rest of a sector a partial write
+    // leaves (measured on the porous box: about 130 MB of DRAM reads per
+    // launch at 128^3).
+    const uint32_t g = (i - (threadIdx.x & 31) * NV) >> 5, gl = (uint32_t)((a.N - 1) >> 5);
+    uint8_t c = a.wcls[min(g, gl)];
+    if (NV == 2) {
+      const uint8_t c1 = a.wcls[min(g + 1, gl)];
+      c = c == c1 ? c : (uint8_t)WCLS_MIXED;
+    }
+    work = inrange && c != WCLS_SOLID;
+    mixed = c == WCLS_MIXED;
+    if (work && mixed) {
+      if constexpr (NV == 2) {
+        const uint2 w = *reinterpret_cast<const uint2*>(a.links + i);
+        lk[0] = w.x;
+        lk[1] = w.y;
+      } else {
+        lk[0] = a.links[i];
+      }
+    }
   }
-  // Wall nodes in a warp with fluid nodes run the same instructions with
-  // their loads switched off and store what they computed from zeros into
-  // their own slots (which no pull reads): every store of the warp then
-  // covers whole sectors, so the L2 need not fetch the rest of a sector a
-  // partial write leaves (measured on the porous box: about 130 MB of DRAM
-  // reads per launch at 128^3).  A warp of wall nodes only does nothing.
-  const bool any_fluid = WALLS ? __any_sync(0xffffffffu, active) : true;  // every lane votes
-  const bool work = inrange && any_fluid;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) act[k] = work && !(lk[k] & LINK_SOLID);
   if (work) {
     int x, y, z;
     site_xyz(i, a.nx, a.ny, x, y, z);
-    const Nbr o = neighbours(x, y, z, a.nx, a.ny, a.nz);
-    const T* __restrict__ fin = static_cast<const T*>(a.fin);
-    T* __restrict__ fout = static_cast<T*>(a.fout);
+    Nbr o = neighbours(x, y, z, a.nx, a.ny, a.nz);
+    if (NV == 2) o.dxp = x + 2 == a.nx ? -(a.nx - 1) : 1;  // from the second node
     const int64_t N = a.N;
-
     // stored h_p = (f_p - w_p n_ref) / (w_p n_ref) of every species, pulled
-    // from r - c_p.  The addresses do not wait for the link word: every
-    // lane loads from its upstream nodes at once; then, in a warp with a
-    // fluid node next to a wall, the directions whose upstream node is a
-    // wall node take the node's own reversed value (halfway bounce-back).
-    // Wall lanes compute from zeros.
-    float f[S][Q];
+    // from r - c_p, or where that is a wall node from the node's own reversed
+    // population (halfway bounce-back)
+    Raw<ST, NV> f[S][Q];
+    auto pull_all = [&]() {
 #pragma unroll
-    for (int p = 0; p < Q; ++p) {
-      const int d = upstream(o, p);
+      for (int p = 0; p < Q; ++p) {
+        const int d = (CY(p) == 1 ? o.dym : (CY(p) == -1 ? o.dyp : 0)) +
+                      (CZ(p) == 1 ? o.dzm : (CZ(p) == -1 ? o.dzp : 0));
+        // upstream nodes of the thread's (first) node and of its second one
+        const uint32_t o0 = (uint32_t)((int)i + d + (CX(p) == 1 ? o.dxm : (CX(p) == -1 ? (NV == 2 ? 1 : o.dxp) : 0))) *
+                            (uint32_t)sizeof(T);
+        const uint32_t o1 = (uint32_t)((int)i + d + (CX(p) == 1 ? 0 : 1 + (CX(p) == -1 ? o.dxp : 0))) *
+                            (uint32_t)sizeof(T);
 #pragma unroll
-      for (int s = 0; s < S; ++s) f[s][p] = pull_h<ST, false>(fin, N, s, p, i, d, 0u);
-    }
-    if (WALLS) {
-      const uint32_t wb = active ? (lk & ~LINK_SOLID) : 0u;
-      if (__any_sync(__activemask(), wb != 0u)) {
+        for (int s = 0; s < S; ++s) {
+          const int64_t pl = (int64_t)(s * Q + p) * N;
+          if constexpr (NV == 1) {
+            f[s][p].v = Fmt<ST>::ldh(pop_at<T>(a.fin, pl, o0));
+          } else if (CX(p) == 0) {
+            f[s][p].v = *reinterpret_cast<const uint32_t*>(pop_at<T>(a.fin, pl, o0));
+          } else {
+            f[s][p].v = (uint32_t)*reinterpret_cast<const unsigned short*>(pop_at<T>(a.fin, pl, o0)) |
+                        (uint32_t)*reinterpret_cast<const unsigned short*>(pop_at<T>(a.fin, pl, o1)) << 16;
+          }
+        }
+      }
+    };
+    // the same with the link word choosing the address: one round trip, where
+    // pulls followed by the bounce-back loads took two
+    auto pull_linked = [&]() {
+      if constexpr (NV == 1) {
+        const uint32_t wb = act[0] ? (lk[0] & ~LINK_SOLID) : 0u;
+#pragma unroll
+        for (int p = 0; p < Q; ++p) {
+          const bool bb = p > 0 && ((wb >> p) & 1u);
+          const int64_t e = bb ? (int64_t)OPP(p) * N + i
+                               : (int64_t)p * N + (uint32_t)((int)i + upstream(o, p));
+          const T* ptr = static_cast<const T*>(a.fin) + e;
+#pragma unroll
+          for (int s = 0; s < S; ++s) {
+            const float h = Fmt<ST>::ldh(ptr + (int64_t)(s * Q) * N);
+            f[s][p].v = V<NV>(act[0] ? h : 0.f);
+          }
+        }
+      }
+    };
+    if (WALLS && NV == 1 && mixed) pull_linked();
+    else pull_all();
+    if constexpr (WALLS && NV == 2) {
+      if (mixed) {
+        // reversed values of the pair where a node is next to a wall node;
+        // wall nodes compute from zeros
+        const uint32_t w0 = act[0] ? (lk[0] & ~LINK_SOLID) : 0u, w1 = act[1] ? (lk[1] & ~LINK_SOLID) : 0u;
 #pragma unroll
         for (int p = 1; p < Q; ++p)
+          if (((w0 | w1) >> p) & 1u) {
+            const uint32_t m = ((w0 >> p) & 1u ? 0x0000ffffu : 0u) | ((w1 >> p) & 1u ? 0xffff0000u : 0u);
 #pragma unroll
-          for (int s = 0; s < S; ++s)
-            if ((wb >> p) & 1u) f[s][p] = Fmt<ST>::ldh(fin + (int64_t)(s * Q + OPP(p)) * N + i);
-      }
-      if (!active) {
+            for (int s = 0; s < S; ++s) {
+              const uint32_t r = *reinterpret_cast<const uint32_t*>(
+                  static_cast<const T*>(a.fin) + (int64_t)(s * Q + OPP(p)) * N + i);
+              f[s][p].v = (f[s][p].v & ~m) | (r & m);
+            }
+          }
 #pragma unroll
-        for (int s = 0; s < S; ++s)
+        for (int k = 0; k < NV; ++k)
+          if (!act[k]) {
 #pragma unroll
-          for (int p = 0; p < Q; ++p) f[s][p] = 0.f;
-      }
-    }
-
-    // n = n_ref (1 + sum w h), j = n_ref sum c w h  (sum w = 1, sum w c = 0),
-    // summed per weight class (faces p = 1..6, edges 7..18) so that each
-    // population costs additions only
-    float mh[S], dn[S], n[S], jx[S], jy[S], jz[S];
+            for (int s = 0; s < S; ++s)
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      float sf = 0.f, se = 0.f, xf = 0.f, xe = 0.f, yf = 0.f, ye = 0.f, zf = 0.f, ze = 0.f;
-#pragma unroll
-      for (int p = 1; p < Q; ++p) {
-        const float hp = f[s][p];
-        if (p <= 6) {
-          sf += hp;
-          if (CX(p)) xf += CX(p) * hp;
-          if (CY(p)) yf += CY(p) * hp;
-          if (CZ(p)) zf += CZ(p) * hp;
-        } else {
-          se += hp;
-          if (CX(p)) xe += CX(p) * hp;
-          if (CY(p)) ye += CY(p) * hp;
-          if (CZ(p)) ze += CZ(p) * hp;
-        }
-      }
-      const float m0 = fmaf(WT(0), f[s][0], fmaf(WT(1), sf, WT(7) * se));
-      const float mx = fmaf(WT(1), xf, WT(7) * xe);
-      const float my = fmaf(WT(1), yf, WT(7) * ye);
-      const float mz = fmaf(WT(1), zf, WT(7) * ze);
-      const float r = a.nref[s];
-      mh[s] = m0;
-      dn[s] = r * m0;
-      n[s] = r + dn[s];
-      jx[s] = r * mx;
-      jy[s] = r * my;
-      jz[s] = r * mz;
-      if (DIAG && active && (!(n[s] > 0.f) || !isfinite(n[s]))) qbad = 1.f;
-    }
-
-    float ntot = 0.f, Jx = 0.f, Jy = 0.f, Jz = 0.f;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      ntot += n[s];
-      Jx += jx[s];
-      Jy += jy[s];
-      Jz += jz[s];
-    }
-    const float inv_ntot = 1.0f / ntot;
-    // barycentric velocity (equal masses: mass-weighted = number-weighted)
-    const float ux = Jx * inv_ntot, uy = Jy * inv_ntot, uz = Jz * inv_ntot;
-
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-    if (CHARGED) psi_gradient<WALLS>(a, i, o, lk, gx, gy, gz);
-    const float Ex = -CS2 * gx + a.eext[0];
-    const float Ey = -CS2 * gy + a.eext[1];
-    const float Ez = -CS2 * gz + a.eext[2];
-
-    // number-weighted mean of the drag velocities u^a + F_el^a / 2
-    float zn = 0.f;
-#pragma unroll
-    for (int s = 0; s < S; ++s) zn += a.valence[s] * n[s];
-    const float vbx = (Jx + 0.5f * zn * Ex) * inv_ntot;
-    const float vby = (Jy + 0.5f * zn * Ey) * inv_ntot;
-    const float vbz = (Jz + 0.5f * zn * Ez) * inv_ntot;
-    // pair frequencies: the fractions x_b and x_b v_b of every species
-    float px[PAIR ? S : 1], pxv[PAIR ? S : 1][3];
-    if (PAIR) {
-#pragma unroll
-      for (int b = 0; b < S; ++b) {
-        px[b] = n[b] * inv_ntot;
-        const float hz = 0.5f * a.valence[b] * n[b];
-        pxv[b][0] = (jx[b] + hz * Ex) * inv_ntot;
-        pxv[b][1] = (jy[b] + hz * Ey) * inv_ntot;
-        pxv[b][2] = (jz[b] + hz * Ez) * inv_ntot;
+              for (int p = 0; p < Q; ++p) f[s][p].clear(k);
+          }
       }
     }
-
-    const float om = a.omega_visc;
-    const float omd = a.omega_drag_z ? a.omega_drag_z[z] : a.omega_drag;
-    uint32_t rnd = 0;
-    if (ST != LBM_FP32) rnd = mix32(i * 0x9E3779B9u ^ mix32(a.step_dev ? *a.step_dev : a.step));
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const float inv_n = 1.0f / n[s];
-      const float usx = jx[s] * inv_n, usy = jy[s] * inv_n, usz = jz[s] * inv_n;
-      float Fx, Fy, Fz;
-      if (PAIR)
-        species_force_pair<S>(s, usx, usy, usz, a.valence[s], Ex, Ey, Ez, px, pxv, a, Fx, Fy, Fz);
-      else
-        species_force(usx, usy, usz, a.valence[s], Ex, Ey, Ez, vbx, vby, vbz, omd, Fx, Fy, Fz);
-      const float usq = usx * usx + usy * usy + usz * usz;
-      const float Fu = Fx * ux + Fy * uy + Fz * uz;
-      // In deviations, d*_p = (1 - omega) d_p + [omega phi_p + g_p - omega w_p n_ref]
-      // with, per weight w_p,
-      //   omega phi_p + g_p - omega w_p n_ref
-      //     = w_p [omega dn + n (-1.5 omega |u^a|^2 - 3 F.u
-      //                          + 4.5 omega a^2 + 9 (F.c)(u.c))]      (even in c)
-      //     + w_p n 3 (omega a + F.c)                                 (odd in c)
-      // a = u^a.c (phi_perp in its reduced form, the Appendix expression;
-      // g_p of Eq. ourforc).  Divided by w_p n_ref this updates the stored
-      // h = d / (w_p n_ref) directly: h*_p = (1 - omega) h_p + (even' +/- odd') / n_ref,
-      // with the bracket values even', odd' free of w_p.  Every term is of
-      // the size of the deviations.
-      const float base = n[s] * (-1.5f * om * usq - 3.0f * Fu);
-      const float odn = om * dn[s];
-      const float inr = 1.0f / a.nref[s];
-      // the per-species factors of the bracket values, once per species:
-      // even' = Ce + Ae a^2 + Be (F.c)(u.c), odd' = Do (omega a + F.c)
-      const float nin = n[s] * inr;
-      const float Ae = nin * (4.5f * om), Be = nin * 9.0f, Ce = inr * (odn + base);
-      const float Do = nin * 3.0f, Dom = Do * om;
-      // moving populations first; the rest population then takes
-      // d*_0 = dn - sum_{p>0} d*_p over the stored (rounded) moving values,
-      // i.e. h*_0 = (sum w h - sum_{p>0} w h*_p) / w_0, which holds exactly
-      // in real arithmetic (phi_perp carries mass n, g_p none) and keeps the
-      // rounding of the weights and of 16-bit stores from drifting the
-      // species mass.
-      // Directions come in opposite pairs (p, p+1), c_{p+1} = -c_p: a = u^a.c,
-      // F.c and u.c flip sign, so each pair shares the even part and takes
-      // +/- the odd part.
-      const float omm = 1.0f - om;
-      float moved = 0.f, mjx = 0.f, mjy = 0.f, mjz = 0.f;
-#pragma unroll
-      for (int p = 1; p < Q; p += 2) {
-        const float av = CX(p) * usx + CY(p) * usy + CZ(p) * usz;
-        const float fc = CX(p) * Fx + CY(p) * Fy + CZ(p) * Fz;
-        const float uc = CX(p) * ux + CY(p) * uy + CZ(p) * uz;
-        const float even = fmaf(Ae, av * av, fmaf(Be, fc * uc, Ce));
-        const float odd = fmaf(Dom, av, Do * fc);
-        const float2 hs = Fmt<ST>::sth_sr2(fout + (int64_t)(s * Q + p) * N + i,
-                                           omm * f[s][p] + (even + odd),
-                                           fout + (int64_t)(s * Q + p + 1) * N + i,
-                                           omm * f[s][p + 1] + (even - odd), lcg_next(rnd));
-        moved += WT(p) * (hs.x + hs.y);  // same weight for p and p+1
-        if constexpr (SCAT) {
-          // charge these two stored values carry to r + c_p and r - c_p
-          // (zero for a neutral species)
-          const float kw = a.scat_k[s] * WT(p);
-          scat_add(p, c0, cp, cm, kw * hs.x);
-          scat_add(p + 1, c0, cp, cm, kw * hs.y);
-        }
-        // momentum carried by the pair at the next step: h*_p moves along
-        // c_p unless r + c_p is a wall node (bit p+1), then it is pulled
-        // back along -c_p; h*_{p+1} likewise with bit p
-        if (DIAG) {
-          float mj = hs.x - hs.y;
-          if (WALLS) mj = (((lk >> (p + 1)) & 1u) ? -hs.x : hs.x) - (((lk >> p) & 1u) ? -hs.y : hs.y);
-          if (CX(p)) mjx += CX(p) * WT(p) * mj;
-          if (CY(p)) mjy += CY(p) * WT(p) * mj;
-          if (CZ(p)) mjz += CZ(p) * WT(p) * mj;
-        }
-      }
-      const float h0 = Fmt<ST>::sth_sr(fout + (int64_t)(s * Q) * N + i, (mh[s] - moved) * INV_WT(0),
-                                       lcg_next(rnd));
-      if constexpr (SCAT) c0[GRP(0)] += a.scat_k[s] * WT(0) * h0;
-      if (DIAG && active) {
-        const float r = a.nref[s];
-        qm[s] = r * (WT(0) * h0 + moved);
-        qjx += r * mjx;
-        qjy += r * mjy;
-        qjz += r * mjz;
-      }
-    }
-    if constexpr (SCAT) scatter_charge(a, x, y, z, c0, cp, cm);
+    V<NV> gx(0.f), gy(0.f), gz(0.f);
+    if (CHARGED) psi_gradient_v<NV, WALLS>(a, i, o, lk, mixed, gx, gy, gz);
+    collide_nodes<S, NV, WALLS, CHARGED, ST, DIAG, PAIR, SCAT>(a, i, z, lk, act, f, gx, gy, gz, sc, q);
+    if constexpr (SCAT) scatter_charge(a, x, y, z, sc);
   }
-
 
   // per-CTA partial sums of the diagnostics (inactive threads add zeros)
   if (DIAG) {
-    float q[DIAG_NQ];
-#pragma unroll
-    for (int k = 0; k < DIAG_NQ; ++k) q[k] = 0.f;
-    float qc = 0.f;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      q[s] = qm[s];
-      qc += a.valence[s] * qm[s];
-    }
-    q[MAX_SPECIES + 0] = qjx;
-    q[MAX_SPECIES + 1] = qjy;
-    q[MAX_SPECIES + 2] = qjz;
-    q[MAX_SPECIES + 3] = qc;
-    q[MAX_SPECIES + 4] = qbad;
+    float v[DIAG_NQ];
+    diag_quantities<S>(a, q, v);
     __shared__ float red[8][DIAG_NQ];
 #pragma unroll
     for (int k = 0; k < DIAG_NQ; ++k) {
-      float v = q[k];
       if (k >= S && k < MAX_SPECIES) continue;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
+      for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v[k];
     }
     __syncthreads();
     if (threadIdx.x < DIAG_NQ) {
@@ -386,53 +664,59 @@ __global__ void __launch_bounds__(256) __maxnreg__((collide_maxnreg<S, WALLS, ST
   }
 }
 
+template <int S, bool W, bool C, int ST, bool SC, bool DIAG, bool PAIR>
+cudaError_t launch_one(const StepArgs& a, cudaStream_t st, int threads, int64_t* ctas) {
+  constexpr int NV = LBM_COLLIDE_NODES;
+  *ctas = nblocks(a.N / NV, threads);
+  k_stream_collide<S, NV, W, C, ST, DIAG, PAIR, SC><<<(unsigned)*ctas, threads, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
 template <int S, bool W, bool C, int ST, bool SC>
-cudaError_t launch_sc2(const StepArgs& a, cudaStream_t st, int threads, bool diag) {
-  const unsigned nb = nblocks(a.N, threads);
+cudaError_t launch_nv(const StepArgs& a, cudaStream_t st, int threads, bool diag,
+                      int64_t* ctas) {
   // the pair-frequency drag exists for three or more species (a binary
   // depends on its one cross frequency, which the host passes as omega_drag)
   constexpr bool CAN_PAIR = S >= 3;
-  if (CAN_PAIR && a.pair_on) {
-    if (diag)
-      k_stream_collide<S, W, C, ST, true, CAN_PAIR, SC><<<nb, threads, 0, st>>>(a);
-    else
-      k_stream_collide<S, W, C, ST, false, CAN_PAIR, SC><<<nb, threads, 0, st>>>(a);
-  } else {
-    if (diag)
-      k_stream_collide<S, W, C, ST, true, false, SC><<<nb, threads, 0, st>>>(a);
-    else
-      k_stream_collide<S, W, C, ST, false, false, SC><<<nb, threads, 0, st>>>(a);
-  }
-  return cudaGetLastError();
+  if (CAN_PAIR && a.pair_on)
+    return diag ? launch_one<S, W, C, ST, SC, true, CAN_PAIR>(a, st, threads, ctas)
+                : launch_one<S, W, C, ST, SC, false, CAN_PAIR>(a, st, threads, ctas);
+  return diag ? launch_one<S, W, C, ST, SC, true, false>(a, st, threads, ctas)
+              : launch_one<S, W, C, ST, SC, false, false>(a, st, threads, ctas);
 }
 
 // The charge scatter: a.scat_acc is set by the host only for charged FP32
 // lattices without walls whose nx is a multiple of 32.
 template <int S, bool W, bool C, int ST>
-cudaError_t launch_sc(const StepArgs& a, cudaStream_t st, int threads, bool diag) {
+cudaError_t launch_sc(const StepArgs& a, cudaStream_t st, int threads, bool diag,
+                      int64_t* ctas) {
   if constexpr (!W && C && ST == LBM_FP32) {
-    if (a.scat_acc) return launch_sc2<S, W, C, ST, true>(a, st, threads, diag);
+    if (a.scat_acc) return launch_nv<S, W, C, ST, true>(a, st, threads, diag, ctas);
   }
-  return launch_sc2<S, W, C, ST, false>(a, st, threads, diag);
+  return launch_nv<S, W, C, ST, false>(a, st, threads, diag, ctas);
 }
 
 template <int S, int ST>
-cudaError_t dispatch_wc(const StepArgs& a, bool w, bool c, cudaStream_t st, int t, bool d) {
-  if (w) return c ? launch_sc<S, true, true, ST>(a, st, t, d) : launch_sc<S, true, false, ST>(a, st, t, d);
-  return c ? launch_sc<S, false, true, ST>(a, st, t, d) : launch_sc<S, false, false, ST>(a, st, t, d);
+cudaError_t dispatch_wc(const StepArgs& a, bool w, bool c, cudaStream_t st, int t, bool d,
+                        int64_t* n) {
+  if (w)
+    return c ? launch_sc<S, true, true, ST>(a, st, t, d, n) : launch_sc<S, true, false, ST>(a, st, t, d, n);
+  return c ? launch_sc<S, false, true, ST>(a, st, t, d, n) : launch_sc<S, false, false, ST>(a, st, t, d, n);
 }
 
 }  // namespace
 
 template <>
-cudaError_t collide_dispatch<LBM_COLLIDE_STORAGE>(const StepArgs& a, int S, bool w, bool c,
-                                                  cudaStream_t st, int threads, bool d) {
+cudaError_t collide_dispatch<LBM_COLLIDE_STORAGE, LBM_COLLIDE_NODES>(const StepArgs& a, int S, bool w,
+                                                                     bool c, cudaStream_t st,
+                                                                     int threads, bool d,
+                                                                     int64_t* ctas) {
   constexpr int ST = LBM_COLLIDE_STORAGE;
   switch (S) {
-    case 1: return dispatch_wc<1, ST>(a, w, c, st, threads, d);
-    case 2: return dispatch_wc<2, ST>(a, w, c, st, threads, d);
-    case 3: return dispatch_wc<3, ST>(a, w, c, st, threads, d);
-    case 4: return dispatch_wc<4, ST>(a, w, c, st, threads, d);
+    case 1: return dispatch_wc<1, ST>(a, w, c, st, threads, d, ctas);
+    case 2: return dispatch_wc<2, ST>(a, w, c, st, threads, d, ctas);
+    case 3: return dispatch_wc<3, ST>(a, w, c, st, threads, d, ctas);
+    case 4: return dispatch_wc<4, ST>(a, w, c, st, threads, d, ctas);
   }
   return cudaErrorInvalidValue;
 }

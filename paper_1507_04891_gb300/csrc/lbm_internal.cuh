@@ -105,13 +105,18 @@ __device__ __forceinline__ int64_t f32_to_i64_rn(float f) {
 //   bit 0      node is a wall node
 //   bit p      (p = 1..18) the upstream node r - c_p is a wall node
 constexpr uint32_t LINK_SOLID = 1u;
+// Class of 32 consecutive nodes (a byte each, with the link words): no wall
+// node and no fluid node next to one; wall nodes only; or some of either.
+enum { WCLS_CLEAR = 0, WCLS_SOLID = 1, WCLS_MIXED = 2 };
 
 struct StepArgs {
   const void* fin;
   void* fout;
   const uint32_t* links;   // NULL without walls
+  const uint8_t* wcls;     // class of every 32 nodes; NULL without walls
   const int64_t* psi;      // fixed point, lattice-sized; NULL when neutral
   const float* wallq;      // face charge share of each wall node; may be NULL
+  const float* wallg;      // wall part of the potential's gradient, [3][N]; may be NULL
   int nx, ny, nz;
   int64_t N;
   float omega_visc, omega_drag;
@@ -254,7 +259,9 @@ struct lbm {
   double mass0 = 0.0;
   bool has_walls = false;
   uint32_t* links = nullptr;
+  uint8_t* wcls = nullptr;  // WCLS_* of every 32 nodes
   float* wallq = nullptr;
+  float* wallg = nullptr;  // wall part of the potential's gradient (k_wall_gradient)
   int64_t* wsrc = nullptr;  // 4 pi l_B w_i in fixed point (wall charge of each fluid cell)
   int64_t nfluid = 0;
   lbm_gb300::Poisson ps;
@@ -353,21 +360,25 @@ namespace lbm_gb300 {
 // the work that the last lbm_step queued on a caller's stream.
 cudaError_t own_stream(lbm_t* h);
 
-// ---- lbm_collide.cu (one object per storage format) ----
-// Launches the fused stream/collide of storage format ST from a to a.fout:
-// S species, walls w, charged c, `threads` per CTA, diagnostics variant d.
-// (a.pair_on selects the pair-frequency drag; three or more species).
-template <int ST>
+// ---- lbm_collide.cu (one object per storage format and nodes per thread) ----
+// Launches the fused stream/collide of storage format ST from a to a.fout,
+// NV consecutive x nodes per thread (2: 16-bit formats, nx even): S species,
+// walls w, charged c, `threads` per CTA, diagnostics variant d (a.pair_on
+// selects the pair-frequency drag; three or more species).  *ctas receives
+// the number of CTAs (of the diagnostics partials).
+template <int ST, int NV>
 cudaError_t collide_dispatch(const StepArgs& a, int S, bool w, bool c, cudaStream_t st,
-                             int threads, bool d);
-template <>
-cudaError_t collide_dispatch<LBM_FP32>(const StepArgs&, int, bool, bool, cudaStream_t, int, bool);
-template <>
-cudaError_t collide_dispatch<LBM_FP16_SHIFT>(const StepArgs&, int, bool, bool, cudaStream_t, int,
-                                             bool);
-template <>
-cudaError_t collide_dispatch<LBM_BF16_SHIFT>(const StepArgs&, int, bool, bool, cudaStream_t, int,
-                                             bool);
+                             int threads, bool d, int64_t* ctas);
+#define LBM_DECL_COLLIDE(ST, NV) \
+  template <>                    \
+  cudaError_t collide_dispatch<ST, NV>(const StepArgs&, int, bool, bool, cudaStream_t, int, bool, \
+                                       int64_t*);
+LBM_DECL_COLLIDE(LBM_FP32, 1)
+LBM_DECL_COLLIDE(LBM_FP16_SHIFT, 1)
+LBM_DECL_COLLIDE(LBM_FP16_SHIFT, 2)
+LBM_DECL_COLLIDE(LBM_BF16_SHIFT, 1)
+LBM_DECL_COLLIDE(LBM_BF16_SHIFT, 2)
+#undef LBM_DECL_COLLIDE
 
 // Records the relative residual at the start of a Poisson solve.
 void note_start_residual(lbm_t* h, double rel);
@@ -416,6 +427,8 @@ cudaError_t launch_species_check(lbm_t* h, const double* n0_dev, const double* u
 cudaError_t launch_diag_reduce(lbm_t* h, double* out, const int* iters = nullptr,
                                const double* rel = nullptr);
 cudaError_t launch_links(lbm_t* h, const uint8_t* solid_dev);
+// Fills h->wallg from the link words and h->wallq.
+cudaError_t launch_wall_gradient(lbm_t* h);
 cudaError_t launch_psi_to_double(lbm_t* h, const int64_t* psi, double* out);
 cudaError_t launch_psi_from_double(lbm_t* h, const double* in, int64_t* psi);
 cudaError_t launch_src_from_rho(lbm_t* h, const double* rho_dev);

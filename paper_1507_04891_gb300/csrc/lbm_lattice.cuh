@@ -53,6 +53,69 @@ __host__ __device__ __forceinline__ constexpr float INV_WT(int p) {
 constexpr float CS2 = 1.0f / 3.0f;
 
 // ---------------------------------------------------------------------------
+// One or two nodes per thread: V<1> is a float, V<2> the values of two
+// consecutive x nodes in a register pair, computed with the packed FP32
+// instructions (add, mul, fma .f32x2: two roundings-to-nearest per issue
+// slot).
+// ---------------------------------------------------------------------------
+template <int NV>
+struct V;
+template <>
+struct V<1> {
+  float a;
+  __device__ __forceinline__ V() {}
+  __device__ __forceinline__ V(float x) : a(x) {}
+  __device__ __forceinline__ float get(int) const { return a; }
+  __device__ __forceinline__ void set(int, float x) { a = x; }
+};
+template <>
+struct V<2> {
+  float2 a;
+  __device__ __forceinline__ V() {}
+  __device__ __forceinline__ V(float x) : a(make_float2(x, x)) {}
+  __device__ __forceinline__ V(float2 x) : a(x) {}
+  __device__ __forceinline__ float get(int k) const { return k ? a.y : a.x; }
+  __device__ __forceinline__ void set(int k, float x) {
+    if (k) a.y = x;
+    else a.x = x;
+  }
+};
+__device__ __forceinline__ V<1> operator+(V<1> x, V<1> y) { return x.a + y.a; }
+__device__ __forceinline__ V<1> operator-(V<1> x, V<1> y) { return x.a - y.a; }
+__device__ __forceinline__ V<1> operator*(V<1> x, V<1> y) { return x.a * y.a; }
+__device__ __forceinline__ V<1> vfma(V<1> x, V<1> y, V<1> z) { return fmaf(x.a, y.a, z.a); }
+__device__ __forceinline__ V<2> operator+(V<2> x, V<2> y) { return __fadd2_rn(x.a, y.a); }
+__device__ __forceinline__ V<2> operator-(V<2> x, V<2> y) {
+  float2 d;
+  asm("{.reg .b64 x, y, d;\n\t"
+      "mov.b64 x, {%2, %3};\n\t"
+      "mov.b64 y, {%4, %5};\n\t"
+      "sub.rn.f32x2 d, x, y;\n\t"
+      "mov.b64 {%0, %1}, d;}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(x.a.x), "f"(x.a.y), "f"(y.a.x), "f"(y.a.y));
+  return d;
+}
+__device__ __forceinline__ V<2> operator*(V<2> x, V<2> y) { return __fmul2_rn(x.a, y.a); }
+__device__ __forceinline__ V<2> vfma(V<2> x, V<2> y, V<2> z) { return __ffma2_rn(x.a, y.a, z.a); }
+// 1 / x: the hardware's reciprocal (one ulp) and one Newton step, within an
+// ulp like the rounded division but without its out-of-range path (densities
+// are far from the ends of the range; zero gives NaN, which the density
+// check reports as it does an infinity).
+__device__ __forceinline__ float rcp_hw(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+template <int NV>
+__device__ __forceinline__ V<NV> vrcp(V<NV> x) {
+  V<NV> r;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) r.set(k, rcp_hw(x.get(k)));
+  return vfma(r, vfma(V<NV>(0.f) - x, r, V<NV>(1.f)), r);
+}
+
+// ---------------------------------------------------------------------------
 // Population storage formats.  The 16-bit formats store the relative
 // deviation from the rest state of the species, h = f / (w_p n_ref) - 1, so
 // that dilute ions keep their relative precision.
@@ -82,6 +145,19 @@ struct Fmt<LBM_FP32> {
     *pa = ha;
     *pb = hb;
     return make_float2(ha, hb);
+  }
+  // the same for two consecutive nodes (pa, pb even): ha, hb become the
+  // stored values
+  static __device__ __forceinline__ float2 ldh2(const T* p) {
+    return *reinterpret_cast<const float2*>(p);
+  }
+  static __device__ __forceinline__ void sth_sr22(T* pa, float2& ha, T* pb, float2& hb, uint32_t,
+                                                  uint32_t) {
+    *reinterpret_cast<float2*>(pa) = ha;
+    *reinterpret_cast<float2*>(pb) = hb;
+  }
+  static __device__ __forceinline__ void sth_sr_pair(T* p, float2& h, uint32_t, uint32_t) {
+    *reinterpret_cast<float2*>(p) = h;
   }
 };
 
@@ -128,6 +204,28 @@ struct Fmt<LBM_FP16_SHIFT> {
     const float2 r = __half22float2(*reinterpret_cast<const __half2*>(&v));
     return make_float2(r.y, r.x);  // ha sits in the upper half
   }
+  static __device__ __forceinline__ float2 ldh2(const T* p) {
+    const uint32_t v = *reinterpret_cast<const uint32_t*>(p);
+    return unpack(v);
+  }
+  // two consecutive nodes, random bits r0, r1 of their own (the same
+  // roundings as sth_sr2 of each): the halves regrouped per direction
+  static __device__ __forceinline__ void sth_sr22(T* pa, float2& ha, T* pb, float2& hb, uint32_t r0,
+                                                  uint32_t r1) {
+    const uint32_t v0 = cvt_rs_f16x2(ha.x, hb.x, r0), v1 = cvt_rs_f16x2(ha.y, hb.y, r1);
+    const uint32_t a = __byte_perm(v0, v1, 0x7632), b = __byte_perm(v0, v1, 0x5410);
+    *reinterpret_cast<uint32_t*>(pa) = a;
+    *reinterpret_cast<uint32_t*>(pb) = b;
+    ha = unpack(a);
+    hb = unpack(b);
+  }
+  static __device__ __forceinline__ void sth_sr_pair(T* p, float2& h, uint32_t r0, uint32_t r1) {
+    const uint32_t v0 = cvt_rs_f16x2(h.x, 0.0f, r0), v1 = cvt_rs_f16x2(h.y, 0.0f, r1);
+    const uint32_t a = __byte_perm(v0, v1, 0x7632);
+    *reinterpret_cast<uint32_t*>(p) = a;
+    h = unpack(a);
+  }
+  static __device__ __forceinline__ float2 unpack(uint32_t v) { return __half22float2(*reinterpret_cast<const __half2*>(&v)); }
 };
 template <>
 struct Fmt<LBM_BF16_SHIFT> {
@@ -155,6 +253,28 @@ struct Fmt<LBM_BF16_SHIFT> {
     *reinterpret_cast<unsigned short*>(pb) = (unsigned short)(v & 0xFFFFu);
     return make_float2(__uint_as_float(v & 0xFFFF0000u), __uint_as_float(v << 16));
   }
+  static __device__ __forceinline__ float2 ldh2(const T* p) {
+    const uint32_t v = *reinterpret_cast<const uint32_t*>(p);
+    return unpack(v);
+  }
+  // two consecutive nodes, random bits r0, r1 of their own (the same
+  // roundings as sth_sr2 of each): the halves regrouped per direction
+  static __device__ __forceinline__ void sth_sr22(T* pa, float2& ha, T* pb, float2& hb, uint32_t r0,
+                                                  uint32_t r1) {
+    const uint32_t v0 = cvt_rs_bf16x2(ha.x, hb.x, r0), v1 = cvt_rs_bf16x2(ha.y, hb.y, r1);
+    const uint32_t a = __byte_perm(v0, v1, 0x7632), b = __byte_perm(v0, v1, 0x5410);
+    *reinterpret_cast<uint32_t*>(pa) = a;
+    *reinterpret_cast<uint32_t*>(pb) = b;
+    ha = unpack(a);
+    hb = unpack(b);
+  }
+  static __device__ __forceinline__ void sth_sr_pair(T* p, float2& h, uint32_t r0, uint32_t r1) {
+    const uint32_t v0 = cvt_rs_bf16x2(h.x, 0.0f, r0), v1 = cvt_rs_bf16x2(h.y, 0.0f, r1);
+    const uint32_t a = __byte_perm(v0, v1, 0x7632);
+    *reinterpret_cast<uint32_t*>(p) = a;
+    h = unpack(a);
+  }
+  static __device__ __forceinline__ float2 unpack(uint32_t v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u)); }
 };
 
 // Counter-based random bits for stochastic rounding: one 32-bit mix of the
