@@ -797,6 +797,7 @@ __global__ void __launch_bounds__(256) k_restrict0(
     for (int ky = 0; ky <= cys; ++ky)
       for (int kx = 0; kx <= cxs; ++kx) {
         const int x = (X << cxs) + kx, y = (Y << cys) + ky, z = (Z << czs) + kz;
+        if (x >= b.nx || y >= b.ny || z >= b.nzb) continue;  // an odd extent's last cell
         const uint32_t q = sp_idx(b, x, y, z);
         const uint32_t m = WALLS ? (uint32_t)mask[q] : FACES_OPEN;
         if (m & FACE_SOLID) continue;
@@ -825,6 +826,7 @@ __global__ void __launch_bounds__(256) k_restrict(
     for (int ky = 0; ky <= cys; ++ky)
       for (int kx = 0; kx <= cxs; ++kx) {
         const int xx = (X << cxs) + kx, yy = (Y << cys) + ky, zz = (Z << czs) + kz;
+        if (xx >= f.nx || yy >= f.ny || zz >= f.nz) continue;
         const uint32_t c = ((uint32_t)zz * f.ny + yy) * f.nx + xx;
         const float di = Dinv[c];
         if (di == 0.f) continue;
@@ -882,16 +884,19 @@ __global__ void __launch_bounds__(256) k_prolong(
         v[dz][dy][dx] = (Dinv_c[Jn] != 0.f) ? xc[Jn] : vp;
       }
   // weight of the parent's coordinate and of the side neighbour per axis
-  const float wx[2] = {cxs ? 0.75f : 1.f, cxs ? 0.25f : 0.f};
-  const float wy[2] = {cys ? 0.75f : 1.f, cys ? 0.25f : 0.f};
-  const float wz[2] = {czs ? 0.75f : 1.f, czs ? 0.25f : 0.f};
+  // (the single child at the end of an odd extent takes the parent's)
+  const bool hx2 = cxs && 2 * X + 1 < f.nx, hy2 = cys && 2 * Y + 1 < f.ny,
+             hz2 = czs && 2 * Z + 1 < f.nz;
+  const float wx[2] = {hx2 ? 0.75f : 1.f, hx2 ? 0.25f : 0.f};
+  const float wy[2] = {hy2 ? 0.75f : 1.f, hy2 ? 0.25f : 0.f};
+  const float wz[2] = {hz2 ? 0.75f : 1.f, hz2 ? 0.25f : 0.f};
 #pragma unroll
   for (int kz = 0; kz < 2; ++kz)
 #pragma unroll
     for (int ky = 0; ky < 2; ++ky)
 #pragma unroll
       for (int kx = 0; kx < 2; ++kx) {
-        if (kx > cxs || ky > cys || kz > czs) continue;
+        if ((kx && !hx2) || (ky && !hy2) || (kz && !hz2)) continue;
         float acc = 0.f;
 #pragma unroll
         for (int c = 0; c < 2; ++c)
@@ -927,6 +932,7 @@ __device__ __forceinline__ float restrict_cell(const float* x, const float* rhs,
     for (int ky = 0; ky <= cys; ++ky)
       for (int kx = 0; kx <= cxs; ++kx) {
         const int xx = (X << cxs) + kx, yy = (Y << cys) + ky, zz = (Z << czs) + kz;
+        if (xx >= f.nx || yy >= f.ny || zz >= f.nz) continue;
         const uint32_t c = ((uint32_t)zz * f.ny + yy) * f.nx + xx;
         const float di = Dinv[c];
         if (di == 0.f) continue;
@@ -1129,14 +1135,14 @@ __global__ void __launch_bounds__(256) k_prolong0_zm(
 // Coarse pair interpolated at fine coordinate i along one axis: p0 the
 // parent, p1 the neighbour on the child's side (the parent outside a
 // non-periodic boundary), w0 the parent's weight.
-__device__ __forceinline__ void prol_pair(int i, int n_c, int per, int coarsened,
+__device__ __forceinline__ void prol_pair(int i, int n_f, int n_c, int per, int coarsened,
                                           int& p0, int& p1, float& w0) {
-  if (!coarsened) {
-    p0 = p1 = i;
+  p0 = coarsened ? i >> 1 : i;
+  if (!coarsened || (i == n_f - 1 && !(i & 1))) {  // or the single child of an odd extent
+    p1 = p0;
     w0 = 1.f;
     return;
   }
-  p0 = i >> 1;
   int q = (i & 1) ? p0 + 1 : p0 - 1;
   if (q < 0 || q >= n_c) {
     if (per) q = (q + n_c) % n_c;
@@ -1148,13 +1154,13 @@ __device__ __forceinline__ void prol_pair(int i, int n_c, int per, int coarsened
 
 // Trilinear interpolation of the coarse correction at fine cell (x, y, z).
 __device__ __forceinline__ float prolong_cell(const float* xc, const float* Dinv_c,
-                                             const CL& cl, int x, int y, int z,
+                                             const CL& f, const CL& cl, int x, int y, int z,
                                              int cxs, int cys, int czs) {
   int ax[2], ay[2], az[2];
   float wx0, wy0, wz0;
-  prol_pair(x, cl.nx, cl.px, cxs, ax[0], ax[1], wx0);
-  prol_pair(y, cl.ny, cl.py, cys, ay[0], ay[1], wy0);
-  prol_pair(z, cl.nz, cl.pz, czs, az[0], az[1], wz0);
+  prol_pair(x, f.nx, cl.nx, cl.px, cxs, ax[0], ax[1], wx0);
+  prol_pair(y, f.ny, cl.ny, cl.py, cys, ay[0], ay[1], wy0);
+  prol_pair(z, f.nz, cl.nz, cl.pz, czs, az[0], az[1], wz0);
   const float wx[2] = {wx0, 1.f - wx0}, wy[2] = {wy0, 1.f - wy0},
               wz[2] = {wz0, 1.f - wz0};
   const int parent = (az[0] * cl.ny + ay[0]) * cl.nx + ax[0];
@@ -1269,7 +1275,7 @@ __global__ void __launch_bounds__(1024) k_sub_cycle(const SubHier H, int nu1, in
       if (f.D[c] == 0.f) continue;
       int xx, yy, zz;
       cl_xyz((uint32_t)c, L, xx, yy, zz);
-      f.e[c] += prolong_cell(cv.e, cv.D, C.l, xx, yy, zz, C.cx, C.cy, C.cz);
+      f.e[c] += prolong_cell(cv.e, cv.D, L, C.l, xx, yy, zz, C.cx, C.cy, C.cz);
     }
     __syncthreads();
     smooth(l, nu2);
@@ -1453,17 +1459,28 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
   }
 
   // Coarsen while the level has more than 64 cells and an axis can halve.
+  // An odd extent halves too: its last coarse cell keeps one child.  (While
+  // only even extents halved, a box of 90x50x75 stopped at 45x25x75 cells and
+  // 50 sweeps over them per cycle were the coarse solve, 100 launches: a step
+  // of a ternary mixture took 2.4 to 4.8 ms; now 0.44 ms.)
   int lx = nx, ly = ny, lz = P.nzb;
   int per[3] = {1, 1, P.perz};
   while ((int64_t)lx * ly * lz > 64 && P.lev.size() < 12) {
-    int cx = (lx % 2 == 0 && lx >= 4), cy = (ly % 2 == 0 && ly >= 4),
-        cz = (lz % 2 == 0 && lz >= 4);
+    const int cx = lx >= 4, cy = ly >= 4, cz = lz >= 4;
     if (!cx && !cy && !cz) break;
-    const int Lx = cx ? lx / 2 : lx, Ly = cy ? ly / 2 : ly, Lz = cz ? lz / 2 : lz;
+    const int Lx = cx ? (lx + 1) / 2 : lx, Ly = cy ? (ly + 1) / 2 : ly, Lz = cz ? (lz + 1) / 2 : lz;
     const int64_t n = (int64_t)Lx * Ly * Lz, nf = (int64_t)lx * ly * lz;
     std::vector<float> Kc(3 * n, 0.f);
     std::vector<char> ac(n, 0);
-    const float sc[3] = {cx ? 0.5f : 1.f, cy ? 0.5f : 1.f, cz ? 0.5f : 1.f};
+    // conductance of a fine face that crosses the + face of a coarse cell:
+    // over the distance of the coarse centres, 2 fine cells between cells of
+    // two children
+    auto scale = [](int c, int X, int l, int L) -> float {
+      if (!c) return 1.f;
+      const int Xn = X + 1 == L ? 0 : X + 1;
+      const int w = (2 * X + 1 < l ? 2 : 1) + (2 * Xn + 1 < l ? 2 : 1);
+      return 2.f / (float)w;
+    };
     for (int z = 0; z < lz; ++z)
       for (int y = 0; y < ly; ++y)
         for (int x = 0; x < lx; ++x) {
@@ -1474,9 +1491,9 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
           ac[J] = 1;
           // a fine face crossing the + face of J: the child on the + side
           // of J along that axis (last child), or any child if not coarsened
-          if (!cx || (x & 1)) Kc[J] += sc[0] * Kh[c];
-          if (!cy || (y & 1)) Kc[n + J] += sc[1] * Kh[nf + c];
-          if (!cz || (z & 1)) Kc[2 * n + J] += sc[2] * Kh[2 * nf + c];
+          if (!cx || (x & 1) || x == lx - 1) Kc[J] += scale(cx, X, lx, Lx) * Kh[c];
+          if (!cy || (y & 1) || y == ly - 1) Kc[n + J] += scale(cy, Y, ly, Ly) * Kh[nf + c];
+          if (!cz || (z & 1) || z == lz - 1) Kc[2 * n + J] += scale(cz, Z, lz, Lz) * Kh[2 * nf + c];
         }
     // inner faces of a non-coarsened axis are within J only if coarsened;
     // for a non-coarsened axis every child's + face is the coarse + face.
@@ -1555,10 +1572,10 @@ bool zm_fine(const Box& b) {
 }
 
 // ... and, for the restriction and prolongation, a first coarse level that
-// halves every axis.
+// halves every axis into whole pairs.
 bool zm_coarse(const Poisson& P, const Box& b) {
-  return zm_fine(b) && P.lev.size() > 1 && P.lev[1].coarsened[0] && P.lev[1].coarsened[1] &&
-         P.lev[1].coarsened[2];
+  return zm_fine(b) && b.nzb % 2 == 0 && P.lev.size() > 1 && P.lev[1].coarsened[0] &&
+         P.lev[1].coarsened[1] && P.lev[1].coarsened[2];
 }
 
 constexpr int ZM_PLANES = 8;         // fine planes per thread
