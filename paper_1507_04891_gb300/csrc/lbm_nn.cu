@@ -76,13 +76,6 @@ __device__ __forceinline__ void xyz(int64_t i, const Geo& G, int& x, int& y, int
   y = (int)(t - (int64_t)z * G.ny);
 }
 
-__device__ __forceinline__ int64_t wrap_idx(const Geo& G, int x, int y, int z) {
-  x = (x + G.nx) % G.nx;
-  y = (y + G.ny) % G.ny;
-  z = (z + G.nz) % G.nz;
-  return ((int64_t)z * G.ny + y) * G.nx + x;
-}
-
 // The 27 neighbours of a cell from six wrapped axis offsets (no modulo per
 // tap): offset of (dx, dy, dz) = ox[dx+1] + oy[dy+1] + oz[dz+1].
 struct Taps {
@@ -110,13 +103,13 @@ __device__ __forceinline__ bool fluid_at(const Geo& G, int64_t i) {
 // (A v)_i over open faces (face open iff both cells fluid).
 __device__ float apply_A(const float* v, const Geo& G, int64_t i, int x, int y, int z) {
   const float vc = v[i];
+  const Taps T = taps_of(G, x, y, z);
+  const int d[6] = {T.ox[2], T.ox[0], T.oy[2], T.oy[0], T.oz[2], T.oz[0]};
   float acc = 0.f;
-  const int d[6][3] = {{1, 0, 0}, {-1, 0, 0}, {0, 1, 0}, {0, -1, 0}, {0, 0, 1}, {0, 0, -1}};
 #pragma unroll
   for (int f = 0; f < 6; ++f) {
-    const int64_t j = wrap_idx(G, x + d[f][0], y + d[f][1], z + d[f][2]);
-    if (j == i || !fluid_at(G, j)) continue;
-    acc += vc - v[j];
+    const int64_t j = i + d[f];
+    if (d[f] != 0 && fluid_at(G, j)) acc += vc - v[j];
   }
   return acc;
 }
@@ -166,28 +159,57 @@ __global__ void k_sum_sq(const float* __restrict__ a, int64_t n, double* out) {
   }
 }
 
+// The FP32 kernels of the training pass are instantiated for up to 4, 8 and
+// 16 channels (CM), so that the sums over channels stay in registers; the
+// weights come from shared memory, the channels of one tap side by side.
+// With a run-time channel count the sums lived in local memory and every tap
+// wrapped its index with three divisions (64^3, 8 channels: layer 1 56 us,
+// layer 2 45 us, its transpose 42 us; now 15, 29 and 11 us).
+template <int CM>
+__device__ __forceinline__ void stage_taps(float* w, const float* __restrict__ p, int C, int stride) {
+  // w[o * CM + c] = p[c * stride + o], zero for c >= C
+  for (int k = threadIdx.x; k < 27 * CM; k += blockDim.x) {
+    const int o = k / CM, c = k - o * CM;
+    w[k] = c < C ? p[c * stride + o] : 0.f;
+  }
+}
+
 // Layer 1 (FP32): hid[c][i] = tanh(b1[c] + sum W1[c][ci][o] x_ci(i + o)).
+template <int CM>
 __global__ void __launch_bounds__(256) k_nn_layer1(const float* __restrict__ x0, const float* __restrict__ p,
                                                    int C, Geo G, float* __restrict__ hid) {
+  __shared__ __align__(16) float wx[27 * CM], wm[27 * CM];
+  stage_taps<CM>(wx, p, C, 54);
+  stage_taps<CM>(wm, p + 27, C, 54);
+  __syncthreads();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= G.N) return;
   int x, y, z;
   xyz(i, G, x, y, z);
-  float acc[16];
-  for (int c = 0; c < C; ++c) acc[c] = p[C * 2 * 27 + c];
+  const Taps T = taps_of(G, x, y, z);
+  float acc[CM];
+#pragma unroll
+  for (int c = 0; c < CM; ++c) acc[c] = c < C ? p[C * 2 * 27 + c] : 0.f;
+#pragma unroll
   for (int o = 0; o < 27; ++o) {
-    const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-    const int64_t j = wrap_idx(G, x + dx, y + dy, z + dz);
+    const int64_t j = i + T.ox[o % 3] + T.oy[(o / 3) % 3] + T.oz[o / 9];
     const float a0 = x0[j];
     const float a1 = fluid_at(G, j) ? 1.f : 0.f;
-    for (int c = 0; c < C; ++c) acc[c] += p[(c * 2 + 0) * 27 + o] * a0 + p[(c * 2 + 1) * 27 + o] * a1;
+#pragma unroll
+    for (int c = 0; c < CM; ++c) acc[c] += wx[o * CM + c] * a0 + wm[o * CM + c] * a1;
   }
-  for (int c = 0; c < C; ++c) hid[(int64_t)c * G.N + i] = tanhf(acc[c]);
+#pragma unroll
+  for (int c = 0; c < CM; ++c)
+    if (c < C) hid[(int64_t)c * G.N + i] = tanhf(acc[c]);
 }
 
 // Layer 2 (FP32): y = sum W2[c][o] hid_c(i + o), zero at wall nodes.
+template <int CM>
 __global__ void __launch_bounds__(256) k_nn_layer2(const float* __restrict__ hid, const float* __restrict__ p,
                                                    int C, Geo G, float* __restrict__ y) {
+  __shared__ __align__(16) float w2[27 * CM];
+  stage_taps<CM>(w2, p + C * 2 * 27 + C, C, 27);
+  __syncthreads();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= G.N) return;
   if (!fluid_at(G, i)) {
@@ -196,12 +218,16 @@ __global__ void __launch_bounds__(256) k_nn_layer2(const float* __restrict__ hid
   }
   int x, yy, z;
   xyz(i, G, x, yy, z);
-  const float* W2 = p + C * 2 * 27 + C;
+  const Taps T = taps_of(G, x, yy, z);
+  // channels outside: the taps of one channel are neighbours in the cache
   float acc = 0.f;
-  for (int o = 0; o < 27; ++o) {
-    const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-    const int64_t j = wrap_idx(G, x + dx, yy + dy, z + dz);
-    for (int c = 0; c < C; ++c) acc += W2[c * 27 + o] * hid[(int64_t)c * G.N + j];
+  for (int c = 0; c < C; ++c) {
+    const float* __restrict__ hc = hid + (int64_t)c * G.N + i;
+    float v[27];
+#pragma unroll
+    for (int o = 0; o < 27; ++o) v[o] = hc[T.ox[o % 3] + T.oy[(o / 3) % 3] + T.oz[o / 9]];
+#pragma unroll
+    for (int o = 0; o < 27; ++o) acc += w2[o * CM + c] * v[o];
   }
   y[i] = acc;
 }
@@ -399,84 +425,149 @@ __global__ void k_nn_gy(const float* __restrict__ res, Geo G, const double* __re
 }
 
 // dL/d(pre-activation)_c = (1 - h_c^2) sum_o W2[c][o] gy(i - o).
+template <int CM>
 __global__ void __launch_bounds__(256) k_nn_ga(const float* __restrict__ gy, const float* __restrict__ hid,
                                                const float* __restrict__ p, int C, Geo G,
                                                float* __restrict__ ga) {
+  __shared__ __align__(16) float w2[27 * CM];
+  stage_taps<CM>(w2, p + C * 2 * 27 + C, C, 27);
+  __syncthreads();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= G.N) return;
   int x, yy, z;
   xyz(i, G, x, yy, z);
-  const float* W2 = p + C * 2 * 27 + C;
-  float acc[16];
-  for (int c = 0; c < C; ++c) acc[c] = 0.f;
+  const Taps T = taps_of(G, x, yy, z);
+  float acc[CM];
+#pragma unroll
+  for (int c = 0; c < CM; ++c) acc[c] = 0.f;
+#pragma unroll
   for (int o = 0; o < 27; ++o) {
-    const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-    const int64_t j = wrap_idx(G, x - dx, yy - dy, z - dz);
+    // the opposite tap: i - o
+    const int64_t j = i + T.ox[2 - o % 3] + T.oy[2 - (o / 3) % 3] + T.oz[2 - o / 9];
     const float gj = gy[j];
-    for (int c = 0; c < C; ++c) acc[c] += W2[c * 27 + o] * gj;
+#pragma unroll
+    for (int c = 0; c < CM; ++c) acc[c] += w2[o * CM + c] * gj;
   }
-  for (int c = 0; c < C; ++c) {
-    const float h = hid[(int64_t)c * G.N + i];
-    ga[(int64_t)c * G.N + i] = acc[c] * (1.f - h * h);
-  }
+#pragma unroll
+  for (int c = 0; c < CM; ++c)
+    if (c < C) {
+      const float h = hid[(int64_t)c * G.N + i];
+      ga[(int64_t)c * G.N + i] = acc[c] * (1.f - h * h);
+    }
 }
 
 // Weight gradients as correlations over cells:
 //   g[W1 c,ci,o] = sum_i ga_c(i) x_ci(i + o),  g[b1 c] = sum_i ga_c(i),
 //   g[W2 c,o]    = sum_i gy(i) hid_c(i + o).
-// Each warp takes 32 cells at a time; every product is reduced across the
-// warp and accumulated per CTA in shared memory, then added to g once per CTA.
-__global__ void __launch_bounds__(256) k_nn_wgrad(const float* __restrict__ gy, const float* __restrict__ ga,
-                                                  const float* __restrict__ hid,
-                                                  const float* __restrict__ x0, int C, Geo G,
-                                                  float* __restrict__ g) {
-  extern __shared__ float acc[];  // np floats
-  const int np = C * 2 * 27 + C + C * 27;
-  for (int k = threadIdx.x; k < np; k += blockDim.x) acc[k] = 0.f;
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int warps_total = gridDim.x * (blockDim.x >> 5);
-  const int64_t nwork = (G.N + 31) / 32;
+// A CTA takes one channel c and one tap plane dz (blockIdx.y) and a share of
+// the (z, x block) columns (blockIdx.x); each of its warps takes a run of
+// rows y: lane = cell of a block of 32 x, the warp walks y with the three
+// rows y - 1 .. y + 1 of x0, the mask and hid_c at z + dz in registers, so
+// that a row costs 11 loads for 27 products, each summed per lane in a
+// register.  One reduction per product over the warp and the CTA at the end,
+// then one atomic.  (With a five-step warp sum for every product of every
+// 32 cells, in CTAs of one warp, 64^3 and 8 channels took 4.38 ms; now 55
+// us.)
+constexpr int WG_WARPS = 8;
+
+__global__ void __launch_bounds__(32 * WG_WARPS) k_nn_wgrad(const float* __restrict__ gy,
+                                                            const float* __restrict__ ga,
+                                                            const float* __restrict__ hid,
+                                                            const float* __restrict__ x0, int C,
+                                                            Geo G, int nwork,
+                                                            float* __restrict__ g) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int c = blockIdx.y / 3, dz = blockIdx.y % 3 - 1;
+  const int nx = G.nx, ny = G.ny, nz = G.nz;
+  const int xb = (nx + 31) / 32;
+  const float* __restrict__ gac = ga + (int64_t)c * G.N;
+  const float* __restrict__ hc = hid + (int64_t)c * G.N;
+  float ax[9], am[9], ah[9], ab = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) ax[k] = am[k] = ah[k] = 0.f;
+  const int rows = (ny + WG_WARPS - 1) / WG_WARPS;
+  const int y0 = wid * rows, y1 = min(y0 + rows, ny);
+  for (int wk = blockIdx.x; wk < nwork; wk += gridDim.x) {
+    const int z = wk / xb, x = (wk - z * xb) * 32 + lane;
+    const bool ok = x < nx;
+    const int xc = ok ? x : nx - 1;
+    int zt = z + dz;
+    zt = zt < 0 ? nz - 1 : (zt == nz ? 0 : zt);
+    const int xi[3] = {xc == 0 ? nx - 1 : xc - 1, xc, xc == nx - 1 ? 0 : xc + 1};
+    // rows y - 1 .. y + 2 of the taps' plane: two rows of cells at a time
+    float vx[4][3], vm[4][3], vh[4][3];
+    auto load = [&](int y, float (&px)[3], float (&pm)[3], float (&ph)[3]) {
+      int yw = y < 0 ? ny - 1 : (y >= ny ? y - ny : y);  // y <= ny + 1
+      if (yw >= ny) yw -= ny;
+      const uint32_t row = (uint32_t)(zt * ny + yw) * (uint32_t)nx;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const uint32_t j = row + (uint32_t)xi[d];
+        px[d] = x0[j];
+        pm[d] = (float)(1u - (G.links ? G.links[j] & LINK_SOLID : 0u));
+        ph[d] = hc[j];
+      }
+    };
+    if (y0 < y1) {
+      load(y0 - 1, vx[0], vm[0], vh[0]);
+      load(y0, vx[1], vm[1], vh[1]);
+    }
+    for (int y = y0; y < y1; y += 2) {
+      const bool two = y + 1 < y1;
+      load(y + 1, vx[2], vm[2], vh[2]);
+      load(y + 2, vx[3], vm[3], vh[3]);
+      float ga_i[2], gy_i[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t i = (uint32_t)(z * ny + min(y + u, ny - 1)) * (uint32_t)nx + (uint32_t)xc;
+        const bool in = ok && (u == 0 || two);
+        ga_i[u] = in ? gac[i] : 0.f;
+        gy_i[u] = in ? gy[i] : 0.f;
+      }
+      ab += ga_i[0] + ga_i[1];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            ax[dy * 3 + d] = fmaf(ga_i[u], vx[dy + u][d], ax[dy * 3 + d]);
+            am[dy * 3 + d] = fmaf(ga_i[u], vm[dy + u][d], am[dy * 3 + d]);
+            ah[dy * 3 + d] = fmaf(gy_i[u], vh[dy + u][d], ah[dy * 3 + d]);
+          }
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          vx[dy][d] = vx[dy + 2][d];
+          vm[dy][d] = vm[dy + 2][d];
+          vh[dy][d] = vh[dy + 2][d];
+        }
+    }
+  }
+  __shared__ float red[WG_WARPS][28];
   auto wsum = [](float v) {
+#pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     return v;
   };
-  for (int64_t wk = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); wk < nwork; wk += warps_total) {
-    const int64_t i = wk * 32 + lane;
-    const bool valid = i < G.N;
-    int x = 0, yy = 0, z = 0;
-    if (valid) xyz(i, G, x, yy, z);
-    float gac[16];
-    for (int c = 0; c < C; ++c) gac[c] = valid ? ga[(int64_t)c * G.N + i] : 0.f;
-    const float gyi = valid ? gy[i] : 0.f;
-    for (int c = 0; c < C; ++c) {
-      const float t = wsum(gac[c]);
-      if (lane == 0) acc[C * 2 * 27 + c] += t;
-    }
-    for (int o = 0; o < 27; ++o) {
-      const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-      int64_t j = 0;
-      float a0 = 0.f, a1 = 0.f;
-      if (valid) {
-        j = wrap_idx(G, x + dx, yy + dy, z + dz);
-        a0 = x0[j];
-        a1 = fluid_at(G, j) ? 1.f : 0.f;
-      }
-      for (int c = 0; c < C; ++c) {
-        const float t0 = wsum(gac[c] * a0);
-        const float t1 = wsum(gac[c] * a1);
-        const float hv = valid ? hid[(int64_t)c * G.N + j] : 0.f;
-        const float t2 = wsum(gyi * hv);
-        if (lane == 0) {
-          acc[(c * 2 + 0) * 27 + o] += t0;
-          acc[(c * 2 + 1) * 27 + o] += t1;
-          acc[C * 2 * 27 + C + c * 27 + o] += t2;
-        }
-      }
-    }
+#pragma unroll
+  for (int k = 0; k < 28; ++k) {
+    const float t = wsum(k < 9 ? ax[k] : (k < 18 ? am[k - 9 < 9 ? k - 9 : 0] : (k < 27 ? ah[k >= 18 ? k - 18 : 0] : ab)));
+    if (lane == 0) red[wid][k] = t;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < np; k += blockDim.x) atomicAdd(g + k, acc[k]);
+  if (threadIdx.x < 28) {
+    const int k = threadIdx.x;
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < WG_WARPS; ++w) t += red[w][k];
+    const int o = (dz + 1) * 9 + k % 9;
+    if (k < 9) atomicAdd(g + (c * 2 + 0) * 27 + o, t);
+    else if (k < 18) atomicAdd(g + (c * 2 + 1) * 27 + o, t);
+    else if (k < 27) atomicAdd(g + C * 2 * 27 + C + c * 27 + o, t);
+    else if (dz == 0) atomicAdd(g + C * 2 * 27 + c, t);
+  }
 }
 
 __global__ void k_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1,
@@ -526,19 +617,28 @@ lbm_status loss_grad(lbm_t* h, bool grad, double* loss) {
   const unsigned gr = (unsigned)std::min<int64_t>(b, h->grid_cap);
   LBM_CUDA_TRY(h, cudaMemsetAsync(n.red, 0, 2 * sizeof(double), h->st));
   k_sum_sq<<<gr, 256, 0, h->st>>>(n.x0, G.N, n.red);
-  k_nn_layer1<<<b, 256, 0, h->st>>>(n.x0, n.p, n.C, G, n.hid);
-  k_nn_layer2<<<b, 256, 0, h->st>>>(n.hid, n.p, n.C, G, n.y);
+#define LBM_NN_C(KERNEL, ...)                                               \
+  do {                                                                      \
+    if (n.C <= 4) KERNEL<4><<<b, 256, 0, h->st>>>(__VA_ARGS__);             \
+    else if (n.C <= 8) KERNEL<8><<<b, 256, 0, h->st>>>(__VA_ARGS__);        \
+    else KERNEL<16><<<b, 256, 0, h->st>>>(__VA_ARGS__);                     \
+  } while (0)
+  LBM_NN_C(k_nn_layer1, n.x0, n.p, n.C, G, n.hid);
+  LBM_NN_C(k_nn_layer2, n.hid, n.p, n.C, G, n.y);
   k_nn_res<<<gr, 256, 0, h->st>>>(n.x0, n.y, G, n.res, n.red);
   h->launches += 4;
   if (grad) {
     k_nn_gy<<<b, 256, 0, h->st>>>(n.res, G, n.red, n.gy);
-    k_nn_ga<<<b, 256, 0, h->st>>>(n.gy, n.hid, n.p, n.C, G, n.ga);
+    LBM_NN_C(k_nn_ga, n.gy, n.hid, n.p, n.C, G, n.ga);
     LBM_CUDA_TRY(h, cudaMemsetAsync(n.g, 0, n.np * sizeof(float), h->st));
-    // CTAs of one warp: lane 0 alone writes the CTA's shared accumulators
-    k_nn_wgrad<<<(unsigned)std::min<int64_t>(nb(G.N, 32), 152), 32, n.np * sizeof(float), h->st>>>(
-        n.gy, n.ga, n.hid, n.x0, n.C, G, n.g);
+    // a few waves of CTAs, at most one per column of 32 x
+    const int nwork = G.nz * ((G.nx + 31) / 32);
+    const int per = std::max(1, std::min(nwork, (2 * h->grid_cap + 3 * n.C - 1) / (3 * n.C)));
+    k_nn_wgrad<<<dim3((unsigned)per, (unsigned)(3 * n.C)), 32 * WG_WARPS, 0, h->st>>>(
+        n.gy, n.ga, n.hid, n.x0, n.C, G, nwork, n.g);
     h->launches += 3;
   }
+#undef LBM_NN_C
   LBM_CUDA_TRY(h, cudaGetLastError());
   LBM_CUDA_TRY(h, cudaMemcpyAsync(n.hred, n.red, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->st));
   LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));
