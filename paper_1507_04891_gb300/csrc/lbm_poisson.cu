@@ -781,26 +781,40 @@ __global__ void __launch_bounds__(256) k_smooth(float* __restrict__ x,
   gs_cell(x, rhs, K, Dinv, l, c, xx, yy, zz);
 }
 
+// Sum of eight lanes' child residuals in the order of the children, kept by
+// every lane of the group (lanes 8 g .. 8 g + 7 belong to one coarse cell).
+__device__ __forceinline__ float child_sum(float v) {
+  const int g = threadIdx.x & 24;
+  float acc = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc += __shfl_sync(0xffffffffu, v, g + k);
+  return acc;
+}
+
 // Restriction from the fine box: rhs_c(J) = sum over the children i of J of
-// (r_i - (A e)_i).
+// (r_i - (A e)_i).  Eight threads per coarse cell J, one per child (bits 0, 1
+// and 2 of the lane: x, y, z): the levels are small and the kernels bound by
+// latency, and one thread walked its eight children one round trip after
+// another (32^3 -> 16^3: 11.3 us in ncu, 64^3 -> 32^3: 13.8; now 4.3 and
+// 6.2).  The children of an axis that is not halved, and the second one of
+// an odd extent's last cell, add zeros.
 template <bool WALLS>
 __global__ void __launch_bounds__(256) k_restrict0(
     const float* __restrict__ e, const float* __restrict__ r,
     const uint8_t* __restrict__ mask, Box b, CL cl, int cxs, int cys,
     int czs, float* __restrict__ rhs_c) {
-  const uint32_t J = blockIdx.x * blockDim.x + threadIdx.x;
-  if (J >= (uint32_t)cl.n) return;
-  int X, Y, Z;
-  cl_xyz(J, cl, X, Y, Z);
-  float acc = 0.f;
-  for (int kz = 0; kz <= czs; ++kz)
-    for (int ky = 0; ky <= cys; ++ky)
-      for (int kx = 0; kx <= cxs; ++kx) {
-        const int x = (X << cxs) + kx, y = (Y << cys) + ky, z = (Z << czs) + kz;
-        if (x >= b.nx || y >= b.ny || z >= b.nzb) continue;  // an odd extent's last cell
-        const uint32_t q = sp_idx(b, x, y, z);
-        const uint32_t m = WALLS ? (uint32_t)mask[q] : FACES_OPEN;
-        if (m & FACE_SOLID) continue;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t J = t >> 3;
+  const int kx = (int)t & 1, ky = (int)(t >> 1) & 1, kz = (int)(t >> 2) & 1;
+  float v = 0.f;
+  if (J < cl.n && kx <= cxs && ky <= cys && kz <= czs) {
+    int X, Y, Z;
+    cl_xyz((uint32_t)J, cl, X, Y, Z);
+    const int x = (X << cxs) + kx, y = (Y << cys) + ky, z = (Z << czs) + kz;
+    if (x < b.nx && y < b.ny && z < b.nzb) {
+      const uint32_t q = sp_idx(b, x, y, z);
+      const uint32_t m = WALLS ? (uint32_t)mask[q] : FACES_OPEN;
+      if (!(m & FACE_SOLID)) {
         uint32_t j[6];
         sp_nbrs(b, x, y, z, j);
         const float ec = e[q];
@@ -808,34 +822,42 @@ __global__ void __launch_bounds__(256) k_restrict0(
 #pragma unroll
         for (int f = 0; f < 6; ++f)
           if ((m >> f) & 1u) Ae += ec - e[j[f]];
-        acc += r[q] - Ae;
+        v = r[q] - Ae;
       }
-  rhs_c[J] = acc;
+    }
+  }
+  v = child_sum(v);
+  if (J < cl.n && (t & 7) == 0) rhs_c[J] = v;
+}
+
+// Residual of child k (bits as above) of coarse cell J on the finer level f,
+// rhs - A x; 0 for a child that is not there or not active.
+__device__ __forceinline__ float child_residual(const float* x, const float* rhs, const float* K,
+                                                const float* Dinv, const CL& f, const CL& cl,
+                                                uint32_t J, int k, int cxs, int cys, int czs) {
+  const int kx = k & 1, ky = (k >> 1) & 1, kz = (k >> 2) & 1;
+  if (kx > cxs || ky > cys || kz > czs) return 0.f;
+  int X, Y, Z;
+  cl_xyz(J, cl, X, Y, Z);
+  const int xx = (X << cxs) + kx, yy = (Y << cys) + ky, zz = (Z << czs) + kz;
+  if (xx >= f.nx || yy >= f.ny || zz >= f.nz) return 0.f;
+  const uint32_t c = ((uint32_t)zz * f.ny + yy) * f.nx + xx;
+  const float di = Dinv[c];
+  if (di == 0.f) return 0.f;
+  int d[6];
+  cl_nbr(f, xx, yy, zz, d);
+  return rhs[c] - (x[c] / di - cl_nsum(x, K, f, c, xx, yy, zz, d));
 }
 
 __global__ void __launch_bounds__(256) k_restrict(
     const float* __restrict__ x, const float* __restrict__ rhs,
     const float* __restrict__ K, const float* __restrict__ Dinv, CL f, CL cl,
     int cxs, int cys, int czs, float* __restrict__ rhs_c) {
-  const uint32_t J = blockIdx.x * blockDim.x + threadIdx.x;
-  if (J >= (uint32_t)cl.n) return;
-  int X, Y, Z;
-  cl_xyz(J, cl, X, Y, Z);
-  float acc = 0.f;
-  for (int kz = 0; kz <= czs; ++kz)
-    for (int ky = 0; ky <= cys; ++ky)
-      for (int kx = 0; kx <= cxs; ++kx) {
-        const int xx = (X << cxs) + kx, yy = (Y << cys) + ky, zz = (Z << czs) + kz;
-        if (xx >= f.nx || yy >= f.ny || zz >= f.nz) continue;
-        const uint32_t c = ((uint32_t)zz * f.ny + yy) * f.nx + xx;
-        const float di = Dinv[c];
-        if (di == 0.f) continue;
-        int d[6];
-        cl_nbr(f, xx, yy, zz, d);
-        const float Ax = x[c] / di - cl_nsum(x, K, f, c, xx, yy, zz, d);
-        acc += rhs[c] - Ax;
-      }
-  rhs_c[J] = acc;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t J = t >> 3;
+  const float v = child_sum(
+      J < cl.n ? child_residual(x, rhs, K, Dinv, f, cl, (uint32_t)J, (int)t & 7, cxs, cys, czs) : 0.f);
+  if (J < cl.n && (t & 7) == 0) rhs_c[J] = v;
 }
 
 // Coarse coordinates along one axis for the prolongation: [0] the neighbour
@@ -849,98 +871,6 @@ __device__ __forceinline__ void prol_axis(int X, int n_c, int per, int coarsened
   else if (per) c[0] = n_c - 1;
   if (X < n_c - 1) c[2] = X + 1;
   else if (per) c[2] = 0;
-}
-
-// Trilinear (cell-centred) prolongation of the coarse correction, added to
-// the fine correction; one thread per coarse cell J writes its children.
-// Along an axis the coarse level halves, child k of J takes 3/4 of J's
-// coordinate and 1/4 of the neighbour on its side (k = 0 below, k = 1
-// above); an inactive coarse cell contributes the parent's value instead.
-// FINE0: the fine level is the fine box (colour-split, face mask);
-// otherwise a level in natural order, Dinv_f = 0 marking inactive cells.
-template <bool FINE0, bool WALLS>
-__global__ void __launch_bounds__(256) k_prolong(
-    float* __restrict__ ef, const float* __restrict__ Dinv_f,
-    const uint8_t* __restrict__ mask, Box b, CL f, const float* __restrict__ xc,
-    const float* __restrict__ Dinv_c, CL cl, int cxs, int cys, int czs) {
-  const uint32_t J = blockIdx.x * blockDim.x + threadIdx.x;
-  if (J >= (uint32_t)cl.n) return;
-  int X, Y, Z;
-  cl_xyz(J, cl, X, Y, Z);
-  int ax[3], ay[3], az[3];
-  prol_axis(X, cl.nx, cl.px, cxs, ax);
-  prol_axis(Y, cl.ny, cl.py, cys, ay);
-  prol_axis(Z, cl.nz, cl.pz, czs, az);
-  const float vp = xc[J];
-  float v[3][3][3];
-#pragma unroll
-  for (int dz = 0; dz < 3; ++dz)
-#pragma unroll
-    for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-      for (int dx = 0; dx < 3; ++dx) {
-        const uint32_t Jn = ((uint32_t)az[dz] * (uint32_t)cl.ny + (uint32_t)ay[dy]) * (uint32_t)cl.nx +
-                            (uint32_t)ax[dx];
-        v[dz][dy][dx] = (Dinv_c[Jn] != 0.f) ? xc[Jn] : vp;
-      }
-  // weight of the parent's coordinate and of the side neighbour per axis
-  // (the single child at the end of an odd extent takes the parent's)
-  const bool hx2 = cxs && 2 * X + 1 < f.nx, hy2 = cys && 2 * Y + 1 < f.ny,
-             hz2 = czs && 2 * Z + 1 < f.nz;
-  const float wx[2] = {hx2 ? 0.75f : 1.f, hx2 ? 0.25f : 0.f};
-  const float wy[2] = {hy2 ? 0.75f : 1.f, hy2 ? 0.25f : 0.f};
-  const float wz[2] = {hz2 ? 0.75f : 1.f, hz2 ? 0.25f : 0.f};
-#pragma unroll
-  for (int kz = 0; kz < 2; ++kz)
-#pragma unroll
-    for (int ky = 0; ky < 2; ++ky)
-#pragma unroll
-      for (int kx = 0; kx < 2; ++kx) {
-        if ((kx && !hx2) || (ky && !hy2) || (kz && !hz2)) continue;
-        float acc = 0.f;
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-          for (int bb = 0; bb < 2; ++bb)
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-              const int sz = c ? (kz ? 2 : 0) : 1, sy = bb ? (ky ? 2 : 0) : 1,
-                        sx = a ? (kx ? 2 : 0) : 1;
-              acc = fmaf(wx[a] * wy[bb] * wz[c], v[sz][sy][sx], acc);
-            }
-        const int x = (X << cxs) + kx, y = (Y << cys) + ky, z = (Z << czs) + kz;
-        if (FINE0) {
-          const uint32_t q = sp_idx(b, x, y, z);
-          if (WALLS && (mask[q] & FACE_SOLID)) continue;
-          ef[q] += acc;
-        } else {
-          const uint32_t c = ((uint32_t)z * (uint32_t)f.ny + (uint32_t)y) * (uint32_t)f.nx + (uint32_t)x;
-          if (Dinv_f[c] == 0.f) continue;
-          ef[c] += acc;
-        }
-      }
-}
-
-// Restricted residual of one coarse cell J: sum over its children i of
-// (rhs_i - (A x)_i) on the finer level f.
-__device__ __forceinline__ float restrict_cell(const float* x, const float* rhs,
-                                              const float* K, const float* Dinv,
-                                              const CL& f, int X, int Y, int Z,
-                                              int cxs, int cys, int czs) {
-  float acc = 0.f;
-  for (int kz = 0; kz <= czs; ++kz)
-    for (int ky = 0; ky <= cys; ++ky)
-      for (int kx = 0; kx <= cxs; ++kx) {
-        const int xx = (X << cxs) + kx, yy = (Y << cys) + ky, zz = (Z << czs) + kz;
-        if (xx >= f.nx || yy >= f.ny || zz >= f.nz) continue;
-        const uint32_t c = ((uint32_t)zz * f.ny + yy) * f.nx + xx;
-        const float di = Dinv[c];
-        if (di == 0.f) continue;
-        int d[6];
-        cl_nbr(f, xx, yy, zz, d);
-        acc += rhs[c] - (x[c] / di - cl_nsum(x, K, f, c, xx, yy, zz, d));
-      }
-  return acc;
 }
 
 // Restriction from the fine box when the coarse level halves every axis
@@ -1152,7 +1082,11 @@ __device__ __forceinline__ void prol_pair(int i, int n_f, int n_c, int per, int 
   w0 = 0.75f;
 }
 
-// Trilinear interpolation of the coarse correction at fine cell (x, y, z).
+// Trilinear (cell-centred) interpolation of the coarse correction at fine
+// cell (x, y, z): along an axis the coarse level halves 3/4 of the parent and
+// 1/4 of the coarse neighbour on the child's side (the single child of an
+// odd extent's last cell: the parent); an inactive coarse cell contributes
+// the parent's value instead.
 __device__ __forceinline__ float prolong_cell(const float* xc, const float* Dinv_c,
                                              const CL& f, const CL& cl, int x, int y, int z,
                                              int cxs, int cys, int czs) {
@@ -1163,21 +1097,48 @@ __device__ __forceinline__ float prolong_cell(const float* xc, const float* Dinv
   prol_pair(z, f.nz, cl.nz, cl.pz, czs, az[0], az[1], wz0);
   const float wx[2] = {wx0, 1.f - wx0}, wy[2] = {wy0, 1.f - wy0},
               wz[2] = {wz0, 1.f - wz0};
-  const int parent = (az[0] * cl.ny + ay[0]) * cl.nx + ax[0];
-  const float vp = xc[parent];
+  float v[8], act[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const uint32_t J = ((uint32_t)az[k >> 2] * (uint32_t)cl.ny + (uint32_t)ay[(k >> 1) & 1]) * (uint32_t)cl.nx +
+                       (uint32_t)ax[k & 1];
+    v[k] = xc[J];
+    act[k] = Dinv_c[J];
+  }
   float acc = 0.f;
 #pragma unroll
-  for (int kz = 0; kz < 2; ++kz)
-#pragma unroll
-    for (int ky = 0; ky < 2; ++ky)
-#pragma unroll
-      for (int kx = 0; kx < 2; ++kx) {
-        const float w = wx[kx] * wy[ky] * wz[kz];
-        if (w == 0.f) continue;
-        const int J = (az[kz] * cl.ny + ay[ky]) * cl.nx + ax[kx];
-        acc += w * ((Dinv_c[J] != 0.f) ? xc[J] : vp);
-      }
+  for (int k = 0; k < 8; ++k)
+    acc = fmaf(wx[k & 1] * wy[(k >> 1) & 1] * wz[k >> 2], act[k] != 0.f ? v[k] : v[0], acc);
   return acc;
+}
+
+// Prolongation, added to the fine correction; one thread per fine cell.
+// FINE0: the fine level is the fine box (colour-split, face mask);
+// otherwise a level in natural order, Dinv_f = 0 marking inactive cells.
+// Latency-bound on the small levels: one thread per coarse cell loaded its
+// 27 neighbours and then read and wrote its children (16^3 -> 32^3: 8.1 us in
+// ncu, 32^3 -> 64^3: 8.7; now 4.3 and 5.4).
+template <bool FINE0, bool WALLS>
+__global__ void __launch_bounds__(256) k_prolong(
+    float* __restrict__ ef, const float* __restrict__ Dinv_f,
+    const uint8_t* __restrict__ mask, Box b, CL f, const float* __restrict__ xc,
+    const float* __restrict__ Dinv_c, CL cl, int cxs, int cys, int czs) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= f.n) return;
+  const uint32_t c = (uint32_t)t;
+  int x, y, z;
+  cl_xyz(c, f, x, y, z);
+  uint32_t q = c;
+  bool on;
+  if (FINE0) {
+    q = sp_idx(b, x, y, z);
+    on = !(WALLS && (mask[q] & FACE_SOLID));
+  } else {
+    on = Dinv_f[c] != 0.f;
+  }
+  const float ev = ef[q];
+  const float add = prolong_cell(xc, Dinv_c, f, cl, x, y, z, cxs, cys, czs);
+  if (on) ef[q] = ev + add;
 }
 
 constexpr int SUB_MAX_LEVELS = 8;
@@ -1196,9 +1157,83 @@ struct SubHier {
   float* e_out;         // its correction (global)
 };
 
+// Sweeps on a coarsest level of at most 64 cells by one warp: a lane keeps
+// its two cells' right-hand side, conductances and neighbour positions in
+// registers and only the corrections go through shared memory, so that a
+// half-sweep is one read, six multiply-adds and one write between two warp
+// barriers.  (By the whole CTA, which found the cells' places by division and
+// read the conductances again in every half-sweep between block barriers,
+// the 100 half-sweeps were about half of k_sub_cycle.)
+__device__ __forceinline__ void bottom_sweeps(float* e, const float* rhs, const float* K,
+                                              const float* D, const CL& L, int sweeps) {
+  const int lane = threadIdx.x & 31;
+  const int n = (int)L.n;
+  const bool compact = L.nx % 2 == 0;  // slot = colour; else cells lane, lane + 32
+  int c[2], col[2], j[2][6];
+  float k[2][6], dv[2], rv[2];
+  bool on[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    uint32_t cc = 0;
+    int x = 0, y = 0, z = 0;
+    if (compact) {
+      on[s] = rb_cell((uint32_t)lane, L.nx, L.ny, L.n, s, true, cc, x, y, z);
+    } else {
+      cc = (uint32_t)(lane + 32 * s);
+      on[s] = (int)cc < n;
+      if (!on[s]) cc = 0;
+      cl_xyz(cc, L, x, y, z);
+    }
+    col[s] = (x + y + z) & 1;
+    c[s] = (int)cc;
+    int d[6];
+    cl_nbr(L, x, y, z, d);
+#pragma unroll
+    for (int f = 0; f < 6; ++f) j[s][f] = c[s] + d[f];
+    k[s][0] = K[c[s]];
+    k[s][1] = K[n + c[s]];
+    k[s][2] = K[2 * n + c[s]];
+    k[s][3] = (L.px || x > 0) ? K[j[s][1]] : 0.f;
+    k[s][4] = (L.py || y > 0) ? K[n + j[s][3]] : 0.f;
+    k[s][5] = (L.pz || z > 0) ? K[2 * n + j[s][5]] : 0.f;
+    dv[s] = D[c[s]];
+    rv[s] = rhs[c[s]];
+    on[s] = on[s] && dv[s] != 0.f;
+  }
+  auto value = [&](int s) {  // the order of cl_nsum
+    float t = k[s][0] * e[j[s][0]];
+    t = fmaf(k[s][1], e[j[s][2]], t);
+    t = fmaf(k[s][2], e[j[s][4]], t);
+    t = fmaf(k[s][3], e[j[s][1]], t);
+    t = fmaf(k[s][4], e[j[s][3]], t);
+    t = fmaf(k[s][5], e[j[s][5]], t);
+    return dv[s] * (rv[s] + t);
+  };
+  for (int it = 0; it < sweeps; ++it) {
+#pragma unroll
+    for (int color = 0; color < 2; ++color) {
+      if (compact) {
+        const float v = value(color);
+        __syncwarp();
+        if (on[color]) e[c[color]] = v;
+      } else {
+        const float v0 = value(0), v1 = value(1);
+        __syncwarp();
+        if (on[0] && col[0] == color) e[c[0]] = v0;
+        if (on[1] && col[1] == color) e[c[1]] = v1;
+      }
+      __syncwarp();
+    }
+  }
+}
+
 // The whole V-cycle below and including a level of at most 4096 cells, in
 // one CTA, every array in shared memory: smoothing, restriction, the
 // coarsest-level sweeps and prolongation, separated by __syncthreads.
+// Latency- and issue-bound (one SM): the places of a thread's cells are found
+// once per smoothing call instead of once per half-sweep, a coarse cell's
+// children are restricted by eight lanes, and one warp does the coarsest
+// level (bottom_sweeps).  16^3 cells and below: 58.2 us in ncu, now 41.1.
 __global__ void __launch_bounds__(1024) k_sub_cycle(const SubHier H, int nu1, int nu2,
                                                     int sweeps) {
   extern __shared__ float sm[];
@@ -1228,6 +1263,7 @@ __global__ void __launch_bounds__(1024) k_sub_cycle(const SubHier H, int nu1, in
   for (int l = 0; l < H.nlev; ++l) {
     const int n = (int)H.lev[l].l.n;
     const Lv v = lv(l);
+#pragma unroll 2
     for (int c = tid; c < n; c += nt) {
       v.e[c] = 0.f;
       v.r[c] = l == 0 ? H.rhs_in[c] : 0.f;
@@ -1241,15 +1277,34 @@ __global__ void __launch_bounds__(1024) k_sub_cycle(const SubHier H, int nu1, in
   auto smooth = [&](int l, int count) {
     const CL L = H.lev[l].l;
     const Lv v = lv(l);
-    const int compact = (L.nx % 2 == 0);
-    const int work = compact ? (int)(L.n >> 1) : (int)L.n;
+    const int n = (int)L.n;
+    if (n <= 64) {
+      if (tid < 32) bottom_sweeps(v.e, v.r, v.K, v.D, L, count);
+      __syncthreads();
+      return;
+    }
+    // work item t: compact, the pair of cells (x0, x0 + 1), one of each
+    // colour; else the cell t.  At most 4096 cells (2048 pairs), and the CTA
+    // has a thread per pair up to 1024: at most four items per thread.
+    const bool compact = L.nx % 2 == 0;
+    const int work = compact ? n >> 1 : n;
+    constexpr int QI = 4;
+    int X[QI], Y[QI], Z[QI];
+#pragma unroll
+    for (int q = 0; q < QI; ++q) {
+      const int t = tid + q * nt;
+      X[q] = -1;
+      if (t < work) cl_xyz((uint32_t)(compact ? 2 * t : t), L, X[q], Y[q], Z[q]);
+    }
     for (int k = 0; k < count; ++k)
       for (int color = 0; color < 2; ++color) {
-        for (int t = tid; t < work; t += nt) {
-          uint32_t c;
-          int xx, yy, zz;
-          if (rb_cell((uint32_t)t, L.nx, L.ny, L.n, color, compact, c, xx, yy, zz))
-            gs_cell(v.e, v.r, v.K, v.D, L, c, xx, yy, zz);
+#pragma unroll
+        for (int q = 0; q < QI; ++q) {
+          if (X[q] < 0) continue;
+          const int par = (X[q] + Y[q] + Z[q] + color) & 1;
+          if (!compact && par) continue;
+          const int x = compact ? X[q] + par : X[q];
+          gs_cell(v.e, v.r, v.K, v.D, L, (uint32_t)((Z[q] * L.ny + Y[q]) * L.nx + x), x, Y[q], Z[q]);
         }
         __syncthreads();
       }
@@ -1259,10 +1314,13 @@ __global__ void __launch_bounds__(1024) k_sub_cycle(const SubHier H, int nu1, in
     const SubLevel& C = H.lev[l + 1];
     const Lv f = lv(l), cv = lv(l + 1);
     const CL F = H.lev[l].l;
-    for (int J = tid; J < (int)C.l.n; J += nt) {
-      int X, Y, Z;
-      cl_xyz((uint32_t)J, C.l, X, Y, Z);
-      cv.r[J] = restrict_cell(f.e, f.r, f.K, f.D, F, X, Y, Z, C.cx, C.cy, C.cz);
+    const int work = 8 * (int)C.l.n;
+    for (int t0 = 0; t0 < work; t0 += nt) {  // the same trips in every thread
+      const int t = t0 + tid;
+      const float r = child_sum(
+          t < work ? child_residual(f.e, f.r, f.K, f.D, F, C.l, (uint32_t)(t >> 3), t & 7, C.cx, C.cy, C.cz)
+                   : 0.f);
+      if (t < work && (t & 7) == 0) cv.r[t >> 3] = r;
     }
     __syncthreads();
   }
@@ -1462,11 +1520,16 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
   // An odd extent halves too: its last coarse cell keeps one child.  (While
   // only even extents halved, a box of 90x50x75 stopped at 45x25x75 cells and
   // 50 sweeps over them per cycle were the coarse solve, 100 launches: a step
-  // of a ternary mixture took 2.4 to 4.8 ms; now 0.44 ms.)
+  // of a ternary mixture took 2.4 to 4.8 ms; now 0.41 ms.)  Short axes halve
+  // down to one cell, below the finest level also from two: where they
+  // stopped at two or three, the cells of a long box grew ever longer and a
+  // cycle smoothed little (to 1e-9, 40x5x3: 64 cycles, now 12; 64x3x3: 202,
+  // now 10; 80x10x6: 59, now 11).
   int lx = nx, ly = ny, lz = P.nzb;
   int per[3] = {1, 1, P.perz};
   while ((int64_t)lx * ly * lz > 64 && P.lev.size() < 12) {
-    const int cx = lx >= 4, cy = ly >= 4, cz = lz >= 4;
+    const int least = P.lev.size() == 1 ? 3 : 2;
+    const int cx = lx >= least, cy = ly >= least, cz = lz >= least;
     if (!cx && !cy && !cz) break;
     const int Lx = cx ? (lx + 1) / 2 : lx, Ly = cy ? (ly + 1) / 2 : ly, Lz = cz ? (lz + 1) / 2 : lz;
     const int64_t n = (int64_t)Lx * Ly * Lz, nf = (int64_t)lx * ly * lz;
@@ -1474,9 +1537,11 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
     std::vector<char> ac(n, 0);
     // conductance of a fine face that crosses the + face of a coarse cell:
     // over the distance of the coarse centres, 2 fine cells between cells of
-    // two children
+    // two children; a face between a cell and itself (one cell on a periodic
+    // axis) couples nothing
     auto scale = [](int c, int X, int l, int L) -> float {
       if (!c) return 1.f;
+      if (L == 1) return 0.f;
       const int Xn = X + 1 == L ? 0 : X + 1;
       const int w = (2 * X + 1 < l ? 2 : 1) + (2 * Xn + 1 < l ? 2 : 1);
       return 2.f / (float)w;
@@ -1797,11 +1862,11 @@ cudaError_t vcycle(lbm_t* h) {
       k_restrict0_zm<false><<<zs.grid, zs.block, 0, h->st>>>(P.lev[0].e, P.lev[0].rhs, nullptr, b,
                                                              cl, zs.zc, C.rhs);
     else if (h->has_walls)
-      k_restrict0<true><<<nblocks(C.n, 256), 256, 0, h->st>>>(
+      k_restrict0<true><<<nblocks(8 * C.n, 256), 256, 0, h->st>>>(
           P.lev[0].e, P.lev[0].rhs, P.face, b, cl, C.coarsened[0], C.coarsened[1],
           C.coarsened[2], C.rhs);
     else
-      k_restrict0<false><<<nblocks(C.n, 256), 256, 0, h->st>>>(
+      k_restrict0<false><<<nblocks(8 * C.n, 256), 256, 0, h->st>>>(
           P.lev[0].e, P.lev[0].rhs, nullptr, b, cl, C.coarsened[0], C.coarsened[1],
           C.coarsened[2], C.rhs);
     ++h->launches;
@@ -1812,7 +1877,7 @@ cudaError_t vcycle(lbm_t* h) {
     if ((e = cudaMemsetAsync(L.e, 0, L.n * sizeof(float), h->st)) != cudaSuccess) return e;
     if ((e = smooth_level(h, l, P.nuc1)) != cudaSuccess) return e;
     PoissonLevel& C = P.lev[l + 1];
-    k_restrict<<<nblocks(C.n, 256), 256, 0, h->st>>>(L.e, L.rhs, L.K, L.Dinv, make_cl(L),
+    k_restrict<<<nblocks(8 * C.n, 256), 256, 0, h->st>>>(L.e, L.rhs, L.K, L.Dinv, make_cl(L),
                                                      make_cl(C), C.coarsened[0],
                                                      C.coarsened[1], C.coarsened[2], C.rhs);
     ++h->launches;
@@ -1827,7 +1892,7 @@ cudaError_t vcycle(lbm_t* h) {
   for (int l = last - 1; l >= 0; --l) {
     PoissonLevel& F = P.lev[l];
     PoissonLevel& C = P.lev[l + 1];
-    const unsigned nb = nblocks(C.n, 256);  // one thread per coarse cell
+    const unsigned nb = nblocks(F.n, 256);  // one thread per fine cell
     if (l == 0 && zm_coarse(P, b)) {
       const CL cl = make_cl(C);
       const ZmShape zs = zm_shape(cl.nx, cl.ny, cl.nz, ZM_COARSE_PLANES);
