@@ -3,6 +3,7 @@
 // density, moment gathers, plane sums, FP64 diagnostics, wall links and
 // potential conversions, and the host-side launchers of all of them.
 #include <algorithm>
+#include <type_traits>
 
 #include "lbm_lattice.cuh"
 
@@ -227,14 +228,18 @@ __device__ __forceinline__ void ld4h(const typename Fmt<ST>::T* p, float (&v)[4]
   }
 }
 
-// The charge density of k_charge for lattices without walls and nx a
-// multiple of four, four consecutive nodes of one x row per thread: the
+// The charge density of k_charge for 16-bit formats and nx a multiple of
+// four, four consecutive nodes of one x row per thread: the
 // four upstream values of a direction are one aligned vector load when the
 // direction has no x component, two when it has (the row's wrap included).
 // The same sums in the same order as k_charge, so the source is the same.
-template <int NC, int ST, bool DOTS>
+// Walls: quads of a group of 32 nodes without wall nodes or neighbours (the
+// class byte) run as without walls; the others load their link words and,
+// beside the upstream values, the nodes' own reversed ones, and choose.
+template <int NC, int ST, bool WALLS, bool DOTS>
 __global__ void __launch_bounds__(256) k_charge_quad(
-    const void* fin_v, int64_t* src, long long* part, int nx, int ny, int nz, int64_t N, int4 cs,
+    const void* fin_v, const uint32_t* links, const uint8_t* wcls, const int64_t* wsrc, int64_t* src,
+    long long* part, const int* label, unsigned long long* comp_sum, int nx, int ny, int nz, int64_t N, int4 cs,
     float4 val, float4 nref, float fourpi_lb, long long src_ref, DotsArgs dk) {
   using T = typename Fmt<ST>::T;
   const T* fin = static_cast<const T*>(fin_v);
@@ -262,6 +267,19 @@ __global__ void __launch_bounds__(256) k_charge_quad(
     const int prevq = (x0 == 0) ? nx - 4 : -4;      // the quad before (x0 - 4 .. x0 - 1)
     const int nextq = (x0 + 4 == nx) ? -(nx - 4) : 4;  // the quad after
     float drho[4] = {0.f, 0.f, 0.f, 0.f};
+    uint32_t lk[4] = {0u, 0u, 0u, 0u};
+    bool solid = false, mixed = false;
+    if (WALLS) {
+      const uint8_t cl = wcls[i0 >> 5];
+      solid = cl == WCLS_SOLID;
+      mixed = cl == WCLS_MIXED;
+      if (mixed) {
+        const uint4 w = *reinterpret_cast<const uint4*>(links + i0);
+        lk[0] = w.x; lk[1] = w.y; lk[2] = w.z; lk[3] = w.w;
+      }
+    }
+    // LINKED: with the reversed values
+    auto sums = [&](auto LINKED) {
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       float m0[4] = {0.f, 0.f, 0.f, 0.f};
@@ -284,6 +302,14 @@ __global__ void __launch_bounds__(256) k_charge_quad(
           ld4h<ST>(b + nextq, a);
           v[0] = h[1]; v[1] = h[2]; v[2] = h[3]; v[3] = a[0];
         }
+        if constexpr (decltype(LINKED)::value) {
+          if (p > 0) {
+            float h[4];
+            ld4h<ST>(fin + (int64_t)(sp[c] * Q + OPP(p)) * N + i0, h);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = ((lk[j] >> p) & 1u) ? h[j] : v[j];
+          }
+        }
         const float wn = WT(p) * nr[c];
 #pragma unroll
         for (int j = 0; j < 4; ++j) m0[j] += wn * v[j];
@@ -291,10 +317,26 @@ __global__ void __launch_bounds__(256) k_charge_quad(
 #pragma unroll
       for (int j = 0; j < 4; ++j) drho[j] += vz[c] * m0[j];
     }
+    };
+    if (!WALLS) {
+      sums(std::false_type{});
+    } else if (!solid) {
+      if (mixed) sums(std::true_type{});
+      else sums(std::false_type{});
+    }
     long long sv[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       sv[j] = src_ref + (long long)(fourpi_lb * drho[j] * PSI_SCALE_F);
+      if (WALLS) {
+        const bool fluid = !solid && !(lk[j] & LINK_SOLID);
+        if (wsrc && fluid) sv[j] += wsrc[i0 + j];
+        if (!fluid) sv[j] = 0;
+        if (label && fluid && label[i0 + j] != 0) {
+          atomicAdd(comp_sum + label[i0 + j], (unsigned long long)sv[j]);
+          continue;
+        }
+      }
       acc += sv[j];
     }
     longlong2* d = reinterpret_cast<longlong2*>(src + i0);
@@ -1011,6 +1053,19 @@ int charge_cta(const lbm_t* h) {
   return h->spec && h->has_walls ? std::min(h->charge_threads, nxy) : h->charge_threads;
 }
 
+// Threads of a CTA of the four-node charge pass, 0 where the one-node pass
+// runs.  16-bit storage: the two-byte loads of one node per thread made the
+// pass request-bound (128^3 FP16 55 -> 40.5 us; 64 stacked slits 118 -> 81 us
+// in ncu); in FP32 the one-node pass is faster, 53 against 61 us at 128^3,
+// and choosing by the class byte in it made it slower beside walls (64x64x66
+// slit 11.0 -> 12.0 us).  As above a CTA stays within a plane where the planes' sums are wanted.
+int charge_quad_cta(const lbm_t* h) {
+  if (h->cfg.storage == LBM_FP32 || h->cfg.nx % 4 != 0) return 0;
+  if (!(h->spec && h->has_walls)) return h->charge_threads;
+  const int q = std::min(h->charge_threads, h->cfg.nx * h->cfg.ny / 4);
+  return q >= 32 ? q : 0;
+}
+
 // The charge pass: the source of the current populations into out (the
 // Poisson source, or the scatter's accumulator), per-CTA partial sums into
 // ps.part; returns the number of partials.
@@ -1049,29 +1104,29 @@ int charge_pass(lbm_t* h, int64_t* out) {
                                  h->f[h->cur], h->links, h->wsrc, out, h->ps.part,           \
                                  h->ps.label, h->ps.comp_sum, h->cfg.nx, h->cfg.ny,          \
                                  h->cfg.nz, h->N, cs4, cv4, cr4, k, src_ref, dk)))
-  // 16-bit storage without walls: four nodes per thread (the two-byte
-  // loads of one node per thread made the pass request-bound; in FP32 the
-  // one-node pass is faster, 53 against 61 us at 128^3)
-  const bool quad = !h->has_walls && h->cfg.storage != LBM_FP32 && h->cfg.nx % 4 == 0;
+  const int qt = charge_quad_cta(h);
+  const bool quad = qt > 0;
   int nbq = nb;
-  if (quad) nbq = (int)nblocks(h->N / 4, ct);
+  if (quad) nbq = (int)nblocks(h->N / 4, qt);
   // (not with walls: there the pass's registers grow from 62 to 80 and it
   // lost more than the separate pass cost, 0.18 against 0.12 ms per step on
   // the porous 256^3 box)
   const bool dots = out == h->ps.src && !h->has_walls && charge_dots_args(h, nbq, &dk);
   if (quad) {
-#define LBM_CHARGE_Q1(NC, ST, D)                                                            \
-  k_charge_quad<NC, ST, D><<<nbq, ct, 0, h->st>>>(h->f[h->cur], out, h->ps.part, h->cfg.nx, \
-                                                  h->cfg.ny, h->cfg.nz, h->N, cs4, cv4, cr4,  \
-                                                  k, src_ref, dk)
+#define LBM_CHARGE_Q1(NC, ST, W, D)                                                            \
+  k_charge_quad<NC, ST, W, D><<<nbq, qt, 0, h->st>>>(                                       \
+      h->f[h->cur], h->links, h->wcls, h->wsrc, out, h->ps.part, h->ps.label, h->ps.comp_sum, \
+      h->cfg.nx, h->cfg.ny, h->cfg.nz, h->N, cs4, cv4, cr4, k, src_ref, dk)
 #define LBM_CHARGE_Q(NC)                                                                   \
   do {                                                                                     \
     if (h->cfg.storage == LBM_FP16_SHIFT) {                                                \
-      if (dots) LBM_CHARGE_Q1(NC, LBM_FP16_SHIFT, true);                                   \
-      else LBM_CHARGE_Q1(NC, LBM_FP16_SHIFT, false);                                       \
+      if (h->has_walls) LBM_CHARGE_Q1(NC, LBM_FP16_SHIFT, true, false);                    \
+      else if (dots) LBM_CHARGE_Q1(NC, LBM_FP16_SHIFT, false, true);                       \
+      else LBM_CHARGE_Q1(NC, LBM_FP16_SHIFT, false, false);                                \
     } else {                                                                               \
-      if (dots) LBM_CHARGE_Q1(NC, LBM_BF16_SHIFT, true);                                   \
-      else LBM_CHARGE_Q1(NC, LBM_BF16_SHIFT, false);                                       \
+      if (h->has_walls) LBM_CHARGE_Q1(NC, LBM_BF16_SHIFT, true, false);                    \
+      else if (dots) LBM_CHARGE_Q1(NC, LBM_BF16_SHIFT, false, true);                       \
+      else LBM_CHARGE_Q1(NC, LBM_BF16_SHIFT, false, false);                                \
     }                                                                                      \
   } while (0)
     switch (nc) {
@@ -1127,7 +1182,8 @@ cudaError_t launch_charge(lbm_t* h) {
   } else {
     nbq = charge_pass(h, h->ps.src);
     // wall planes: the source means of the runs (the total is not used)
-    if (h->has_walls && spectral_run_means(h, charge_cta(h))) {
+    const int qt = charge_quad_cta(h);
+    if (h->has_walls && spectral_run_means(h, qt > 0 ? 4 * qt : charge_cta(h))) {
       h->charge_means_ready = true;
       return cudaGetLastError();
     }
