@@ -64,8 +64,16 @@ static_assert(ST_RING == START_RING_IDX, "ring position index shared with the ch
 // relative diagonal load of 1e-10 against rounding, rows and columns from m
 // on replaced by the identity.  Lane i K + j holds entry (i, j), lane
 // K K + i the right-hand side of row i.  Returns false in every lane when a
-// pivot is not positive or a coefficient is not finite; else lane K K + i
-// returns coefficient i.
+// pivot is not positive or a coefficient is beyond COEF_MAX (or not finite);
+// else lane K K + i returns coefficient i.  The differences of a relaxing run
+// become almost dependent, and their inner products are FP32 sums: now and
+// then the smallest pivot was rounding noise, the coefficients grew and the
+// start was so poor that the step needed a second application.  Extrapolation
+// from K = 5 differences has coefficients up to 10.  (Of 48 passes of 20
+// recorded steps at 128x64x64, 4 had such a step without the limit, none
+// with it; heavier loads of the diagonal cost multigrid cycles on the porous
+// box, 3.4 to 4.2 a step against 3.2.)
+constexpr double COEF_MAX = 16.0;
 __device__ bool solve_gram(const double* G, const double* rhs, int m, double& c) {
   const int lane = threadIdx.x & 31;
   const bool mat = lane < K * K;
@@ -90,7 +98,7 @@ __device__ bool solve_gram(const double* G, const double* rhs, int m, double& c)
   // the diagonal is left: row i's right-hand side over it
   const double d = __shfl_sync(0xffffffffu, v, i * K + i);
   c = v / (d != 0.0 ? d : 1.0);
-  ok = ok && (mat || isfinite(c));
+  ok = ok && (mat || fabs(c) <= COEF_MAX);
   return __all_sync(0xffffffffu, ok);
 }
 
