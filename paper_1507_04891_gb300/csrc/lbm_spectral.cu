@@ -929,6 +929,19 @@ __global__ void __launch_bounds__(256, 4) k_res_planes(
   add_norms(acc, rr, ss, red_r, red_s);
 }
 
+// Allows a kernel the largest dynamic shared memory beside its static one.
+// The limit belongs to the kernel, not to a plan: set to one plan's size it
+// would be too small for another's launches (and the default of 48 KB counts
+// the static part: a run of 128 planes asks for 48 KB of dynamic memory).
+template <class Kernel>
+cudaError_t allow_smem(Kernel* k, int optin) {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, k);
+  return e != cudaSuccess ? e
+                          : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 optin - (int)fa.sharedSizeBytes);
+}
+
 int ilog2(int n) {
   int l = 0;
   while ((1 << l) < n) ++l;
@@ -1155,8 +1168,7 @@ lbm_status spectral_setup(lbm_t* h, const uint8_t* solid) {
   }
   // (without walls yet the plan is provisional: set_walls rebuilds it)
   if (s->runs_fit && s->lgz < 0) {
-    if (s->zsmem > 48 * 1024)
-      LBM_CUDA_TRY(h, cudaFuncSetAttribute(k_zsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->zsmem));
+    LBM_CUDA_TRY(h, allow_smem(k_zsolve, optin));
     const int cyclic = runs[0].cyclic;  // a cyclic run is the only one
     if (!al((void**)&s->ztab, (size_t)lmax * s->mxy * sizeof(float)) ||
         (cyclic && !al((void**)&s->qtab, (size_t)lmax * s->mxy * sizeof(float)))) {
@@ -1175,10 +1187,8 @@ lbm_status spectral_setup(lbm_t* h, const uint8_t* solid) {
     h->err = "spectral Poisson solver: x-y plane too large for shared memory";
     return LBM_EINVAL;
   }
-  if (s->plane_smem > 48 * 1024) {
-    LBM_CUDA_TRY(h, cudaFuncSetAttribute(k_plane_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->plane_smem));
-    LBM_CUDA_TRY(h, cudaFuncSetAttribute(k_plane_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->plane_smem));
-  }
+  LBM_CUDA_TRY(h, allow_smem(k_plane_fwd, optin));
+  LBM_CUDA_TRY(h, allow_smem(k_plane_inv, optin));
   return LBM_OK;
 }
 
