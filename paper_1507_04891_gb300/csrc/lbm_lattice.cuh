@@ -98,7 +98,8 @@ __device__ __forceinline__ V<2> operator-(V<2> x, V<2> y) {
 }
 __device__ __forceinline__ V<2> operator*(V<2> x, V<2> y) { return __fmul2_rn(x.a, y.a); }
 __device__ __forceinline__ V<2> vfma(V<2> x, V<2> y, V<2> z) { return __ffma2_rn(x.a, y.a, z.a); }
-// 1 / x: the hardware's reciprocal (one ulp) and one Newton step, within an
+// 1 / x: the hardware's reciprocal estimate (one ulp) and one step of the
+// Newton-Raphson iteration r <- r + r (1 - x r), within an
 // ulp like the rounded division but without its out-of-range path (densities
 // are far from the ends of the range; zero gives NaN, which the density
 // check reports as it does an infinity).
