@@ -233,57 +233,76 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_start_solve(const float* __re
   }
 }
 
+// What the step's bookkeeping after the start reads and writes, and the
+// start's own arrays.
+struct PsiArgs {
+  int64_t* psi;
+  int64_t* psi_prev;
+  float* ring_p;
+  const float* coef;
+  int* skip_out;          // speculation flag of a step graph, or NULL
+  const int* prev_iters;  // the previous step's applications (with skip_out)
+  int kbaked;
+  float* clear;           // norm slot to clear, or NULL
+  int nclear;
+};
+
+// The step's bookkeeping after the start, by one CTA: the terms it used (for
+// the graph's decisions); in a step graph also whether the step speculates
+// and the cleared norm slot of the first application, which saves graph nodes
+// on the step's critical path.  The step does not speculate when the start
+// used fewer than START_FULL_TERMS differences, or when the previous step
+// needed more than the k applications baked into the graph (prev_iters: its
+// count): steps that need more come in runs (the first steps after a restart,
+// a change in the source the history does not follow), and a step that does
+// not speculate only serialises its stream/collide behind the convergence
+// test, while a failed speculation runs the stream/collide twice.
+__device__ __forceinline__ void start_mark(int* __restrict__ state, const PsiArgs& pa) {
+  if (threadIdx.x == 0) {
+    const int used = state[ST_TERMS];
+    state[ST_USED] = used;
+    if (pa.skip_out)
+      *pa.skip_out = (used < START_FULL_TERMS || (pa.prev_iters && *pa.prev_iters > pa.kbaked)) ? 1 : 0;
+  }
+  for (int k = threadIdx.x; k < pa.nclear; k += blockDim.x) pa.clear[k] = 0.f;
+}
+
 // Pass 3: psi(t-1) + sum_j c_j P_j with P_1 = psi(t-1) - psi(t-2) (fresh)
 // and P_j, j >= 2, from the ring (age j in slot (r - j + 1) mod K); psi(t-1)
 // becomes the stored previous potential and P_1 replaces the slot of age
 // K + 1 (slot r mod K).  The correction is formed in FP32 and rounded to the
 // fixed-point grid; one too large for it keeps psi(t-1).
-__global__ void __launch_bounds__(256) k_start_psi(int64_t* __restrict__ psi,
-                                                   int64_t* __restrict__ psi_prev,
-                                                   float* __restrict__ ring_p,
-                                                   const float* __restrict__ coef,
-                                                   int* __restrict__ state, int64_t N,
-                                                   int advance) {
+// mark: CTA 0 also does the bookkeeping (it writes nothing that the start
+// reads).  As a kernel of its own it was a launch on the critical path: slit
+// 64x64x66, 50 steps 4569 -> 4474 us; BF16 64^3 from the host, 20 steps 1996 ->
+// 1917.
+__global__ void __launch_bounds__(256) k_start_psi(int* __restrict__ state, int64_t N, int mark,
+                                                   const PsiArgs pa) {
+  if (mark && blockIdx.x == 0) start_mark(state, pa);
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
   const int r = state[ST_RING];
   const int m = state[ST_TERMS];
-  const int64_t a = psi[i];
-  const float p1 = i64_to_f32(a - psi_prev[i]);
+  const int64_t a = pa.psi[i];
+  const float p1 = i64_to_f32(a - pa.psi_prev[i]);
   if (m > 0) {
-    float corr = coef[0] * p1;
+    float corr = pa.coef[0] * p1;
 #pragma unroll
     for (int j = 2; j <= K; ++j)
-      if (j <= m) corr += coef[j - 1] * ring_p[(int64_t)((r - j + 1 + K) % K) * N + i];
-    if (fabsf(corr) < 2.3e18f) psi[i] = a + f32_to_i64_rn(corr);
+      if (j <= m) corr += pa.coef[j - 1] * pa.ring_p[(int64_t)((r - j + 1 + K) % K) * N + i];
+    if (fabsf(corr) < 2.3e18f) pa.psi[i] = a + f32_to_i64_rn(corr);
   }
-  psi_prev[i] = a;
-  ring_p[(int64_t)(r % K) * N + i] = p1;
+  pa.psi_prev[i] = a;
+  pa.ring_p[(int64_t)(r % K) * N + i] = p1;
 }
 
-// The step's bookkeeping after the start: the terms it used (for the
-// graph's decisions) and, when it is the step's last pass, the ring
-// position; after every thread of the start read them.  In a step graph it
-// also writes whether the step speculates and clears the norm slot of the
-// first application, which saves two graph nodes on the step's critical
-// path.  The step does not speculate when the start used fewer than
-// START_FULL_TERMS differences, or when the previous step needed more than
-// the k applications baked into the graph (prev_iters: its count): steps
-// that need more come in runs (the first steps after a restart, a change
-// in the source the history does not follow), and a step that does not
-// speculate only serialises its stream/collide behind the convergence
-// test, while a failed speculation runs the stream/collide twice.
-__global__ void k_start_mark(int* __restrict__ state, int advance, int* __restrict__ skip_out,
-                             const int* __restrict__ prev_iters, int kbaked,
-                             float* __restrict__ clear, int nclear) {
-  if (threadIdx.x == 0) {
-    const int used = state[ST_TERMS];
-    state[ST_USED] = used;
-    if (advance) state[ST_RING] = (state[ST_RING] + 1) % K;
-    if (skip_out)
-      *skip_out = (used < START_FULL_TERMS || (prev_iters && *prev_iters > kbaked)) ? 1 : 0;
-  }
-  for (int k = threadIdx.x; k < nclear; k += blockDim.x) clear[k] = 0.f;
+// The bookkeeping of a start that is the step's last pass (the fit ran
+// before it): it moves the ring position, after every thread of the start
+// read it.
+__global__ void k_start_mark(int* __restrict__ state, const PsiArgs pa) {
+  start_mark(state, pa);
+  __syncthreads();
+  if (threadIdx.x == 0) state[ST_RING] = (state[ST_RING] + 1) % K;
 }
 
 // The charge scatter's source take fused with pass 1 (the step's source
@@ -300,18 +319,6 @@ __global__ void k_start_mark(int* __restrict__ state, int advance, int* __restri
 // coefficients are known at the step's start), and the last CTA does
 // k_start_mark's bookkeeping (terms used, the speculation flag, the first
 // norm slot cleared; no ring advance: the fit advances it).
-struct PsiArgs {
-  int64_t* psi;
-  int64_t* psi_prev;
-  float* ring_p;
-  const float* coef;
-  int* skip_out;          // speculation flag of a step graph, or NULL
-  const int* prev_iters;  // the previous step's applications (with skip_out)
-  int kbaked;
-  float* clear;           // norm slot to clear, or NULL
-  int nclear;
-};
-
 template <bool PSI>
 __global__ void __launch_bounds__(256) k_take_dots(int64_t* __restrict__ acc,
                                                    int64_t* __restrict__ src,
@@ -420,16 +427,9 @@ __global__ void __launch_bounds__(256) k_take_dots(int64_t* __restrict__ acc,
     *out = td;
     s_mean = llrint(td * inv_nfluid);
     if (step) *step += 1u;
-    if (PSI) {
-      // every CTA read the terms and the ring position before counting itself
-      const int used = state[ST_TERMS];
-      state[ST_USED] = used;
-      if (pa.skip_out)
-        *pa.skip_out = (used < START_FULL_TERMS || (pa.prev_iters && *pa.prev_iters > pa.kbaked)) ? 1 : 0;
-    }
   }
-  if (PSI)
-    for (int k = threadIdx.x; k < pa.nclear; k += blockDim.x) pa.clear[k] = 0.f;
+  // (every CTA read the terms and the ring position before counting itself)
+  if (PSI) start_mark(state, pa);
   if (mean_z) {
     __syncthreads();
     for (int z = threadIdx.x; z < nz; z += blockDim.x) mean_z[z] = s_mean;
@@ -552,12 +552,23 @@ cudaError_t start_apply(lbm_t* h, bool last) {
     return cudaSuccess;
   }
   H.psi_done = false;
-  k_start_psi<<<nblk(h->N, 256), 256, 0, h->st>>>(h->ps.psi[h->ps.cur], H.psi_prev, H.ring_p, H.coef,
-                                                   H.state, h->N, last ? 1 : 0);
-  k_start_mark<<<1, 128, 0, h->st>>>(H.state, last ? 1 : 0, h->mark_skip_out, h->mark_prev_iters,
-                                     h->mark_k, h->mark_clear, h->mark_clear ? h->mark_nclear : 0);
+  PsiArgs pa{};
+  pa.psi = h->ps.psi[h->ps.cur];
+  pa.psi_prev = H.psi_prev;
+  pa.ring_p = H.ring_p;
+  pa.coef = H.coef;
+  pa.skip_out = h->mark_skip_out;
+  pa.prev_iters = h->mark_prev_iters;
+  pa.kbaked = h->mark_k;
+  pa.clear = h->mark_clear;
+  pa.nclear = h->mark_clear ? h->mark_nclear : 0;
+  k_start_psi<<<nblk(h->N, 256), 256, 0, h->st>>>(H.state, h->N, last ? 0 : 1, pa);
+  ++h->launches;
+  if (last) {
+    k_start_mark<<<1, 128, 0, h->st>>>(H.state, pa);
+    ++h->launches;
+  }
   h->slot0_cleared = h->mark_clear != nullptr;
-  h->launches += 2;
   return cudaGetLastError();
 }
 
