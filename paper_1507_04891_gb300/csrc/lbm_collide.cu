@@ -80,10 +80,12 @@ struct Scat {
   }
 };
 
-// Nearest fixed-point integer of a float below 2^62: the part above 2^32
+// Nearest fixed-point integer of a float below 2^63: the part above 2^32
 // (rounded, so that the rest is exact in FP32 and signed) and the rest, each
-// by the 32-bit conversion (a rest of exactly 2^31 loses one unit of 2^-52).
-// Seven instructions; f32_to_i64_rn's shifts of 64-bit words took about
+// by the 32-bit conversion; a rest of 2^31, which the conversion saturates to
+// 2^31 - 1 (no other rest gives that: FP32 steps by 128 there), gets its unit
+// back.
+// Ten instructions; f32_to_i64_rn's shifts of 64-bit words took about
 // three times as many, and the scatter converts 9 to 14 sums per node.
 // With the 32-bit node offsets and the reciprocal of vrcp the kernel with the
 // scatter went from 1.30e8 to 1.06e8 warp instructions at 128^3, 178.6 ->
@@ -91,7 +93,7 @@ struct Scat {
 __device__ __forceinline__ unsigned long long scat_fixed(float c) {
   const int hi = __float2int_rn(c * 2.3283064365386963e-10f);
   const int lo = __float2int_rn(fmaf(-4294967296.0f, (float)hi, c));
-  return (unsigned long long)(((long long)hi << 32) + (long long)lo);
+  return (unsigned long long)(((long long)hi << 32) + (long long)lo + (lo == 0x7fffffff ? 1 : 0));
 }
 
 // A warp holds 32 consecutive nodes of one x row (nx is a multiple of 32).
@@ -137,6 +139,27 @@ __device__ __forceinline__ void scatter_charge(const StepArgs& a, int x, int y, 
                 scat_fixed(lane == 0 ? c.qm[j] : c.qp[j]));
   }
 }
+
+// r + x, node by node: the packed form of r + r * y comes out fused.
+template <int NV>
+__device__ __forceinline__ V<NV> add_scalar(float r, const V<NV>& x) {
+  V<NV> v;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v.set(k, __fadd_rn(r, x.get(k)));
+  return v;
+}
+
+// x * y, formed here even if it was formed before: for one node per thread a
+// value kept from the moments to the update would hold a register in the
+// part of the kernel that has none to spare (ternary 128^3, FP32 with the
+// charge scatter: 172 us a launch with the product kept, 162 with it formed
+// again).
+__device__ __forceinline__ V<1> mul_here(V<1> x, V<1> y) {
+  float r;
+  asm volatile("mul.rn.f32 %0, %1, %2;" : "=f"(r) : "f"(x.a), "f"(y.a));
+  return r;
+}
+__device__ __forceinline__ V<2> mul_here(V<2> x, V<2> y) { return x * y; }
 
 // c . v for the direction p (a constant once unrolled): additions only.
 template <int NV>
@@ -199,19 +222,18 @@ __device__ __forceinline__ const T* pop_at(const void* base, int64_t plane, uint
 }
 
 // Gradient of psi along one axis at a node: mean of the two face gradients,
-// half the difference of the two neighbours between open faces (an exact
-// integer difference, rounded once).  At a wall face the node's own value
-// takes the neighbour's place and the Neumann value of the surface-charge
-// condition is in the wall part w (k_wall_gradient).
+// each an exact integer difference, rounded once (a step of psi up to 2^11
+// per face).  At a wall face the node's own value takes the neighbour's
+// place and the Neumann value of the surface-charge condition is in the wall
+// part w (k_wall_gradient).
 template <bool WALLS>
 __device__ __forceinline__ float axis_gradient(int64_t c, int64_t m, int64_t p, uint32_t wm, uint32_t wp,
                                                float w) {
   if (WALLS) {
     p = wp ? c : p;
     m = wm ? c : m;
-    return fmaf((float)(p - m), 0.5f * PSI_INV_SCALE_F, w);
   }
-  return (float)(p - m) * (0.5f * PSI_INV_SCALE_F);
+  return fmaf((float)(p - c) + (float)(c - m), 0.5f * PSI_INV_SCALE_F, w);
 }
 
 // Potential of NV consecutive nodes.
@@ -233,7 +255,7 @@ __device__ __forceinline__ void psi_gradient_v(const StepArgs& a, uint32_t i, co
                                                V<NV>& gy, V<NV>& gz) {
   const int64_t* __restrict__ ps = a.psi + i;
   int64_t c[NV] = {}, yp[NV], ym[NV], zp[NV], zm[NV];
-  if (WALLS || NV == 2) ld_psi<NV>(ps, c);
+  ld_psi<NV>(ps, c);
   ld_psi<NV>(ps + o.dyp, yp);
   ld_psi<NV>(ps + o.dym, ym);
   ld_psi<NV>(ps + o.dzp, zp);
@@ -257,6 +279,23 @@ __device__ __forceinline__ void psi_gradient_v(const StepArgs& a, uint32_t i, co
   }
 }
 
+// The step's roundings are all written out (no multiplication and addition
+// that the compiler may or may not contract), so that one and two nodes per
+// thread and every instance round alike, and so that runs repeat the results
+// of earlier versions of the library bit for bit: near the tolerance of the
+// Poisson solve one rounding decides how many applications a step takes,
+// which the records hold.  Three places keep a contraction that only some
+// instances had:
+//   total    the densities in the sum over species, charged beside walls
+//   density  the fourth species' density, neutral and periodic in FP32
+//   drag     the mean velocity of a single species in its own drag
+template <int S, bool WALLS, bool CHARGED, int ST, bool DIAG, bool PAIR>
+struct Fused {
+  static constexpr bool total = S > 1 && WALLS && CHARGED && !DIAG && !PAIR;
+  static constexpr bool density3 = S == 4 && ST == LBM_FP32 && !WALLS && !CHARGED && !DIAG && !PAIR;
+  static constexpr bool drag = S == 1 && !(WALLS && CHARGED);
+};
+
 // The collision of a thread's NV nodes from i on (plane z) and the stores:
 // f the pulled h_p, (gx, gy, gz) the potential's gradient, lk the link words
 // and act the fluid flags of the nodes.
@@ -268,28 +307,33 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
                                               Sums<S>& q) {
   using T = typename Fmt<ST>::T;
   using F = V<NV>;
+  using FU = Fused<S, WALLS, CHARGED, ST, DIAG, PAIR>;
   T* __restrict__ fout = static_cast<T*>(a.fout) + i;
   const int64_t N = a.N;
   // n = n_ref (1 + sum w h), j = n_ref sum c w h  (sum w = 1, sum w c = 0),
   // summed per weight class (faces p = 1..6, edges 7..18) so that each
   // population costs additions only
-  F mh[S], n[S], jx[S], jy[S], jz[S];
+  F mh[S], n[S], jx[S], jy[S], jz[S], ntot;
 #pragma unroll
   for (int s = 0; s < S; ++s) {
     F h[Q];
 #pragma unroll
     for (int p = 0; p < Q; ++p) h[p] = f[s][p].get();
-    const F sf = ((h[1] + h[2]) + (h[3] + h[4])) + (h[5] + h[6]);
-    F se = h[7];
+    F sf = h[1], se = h[7];
+#pragma unroll
+    for (int p = 2; p <= 6; ++p) sf = sf + h[p];
 #pragma unroll
     for (int p = 8; p < Q; ++p) se = se + h[p];
-    // x: faces 1 - 2, edges 7 - 8 + 9 - 10 + 11 - 12 + 13 - 14, and so on
-    const F xe = ((h[7] - h[8]) + (h[9] - h[10])) + ((h[11] - h[12]) + (h[13] - h[14]));
-    const F ye = ((h[7] - h[8]) - (h[9] - h[10])) + ((h[15] - h[16]) + (h[17] - h[18]));
-    const F ze = ((h[11] - h[12]) - (h[13] - h[14])) + ((h[15] - h[16]) - (h[17] - h[18]));
+    // edges with an x, y or z component, in the order of the directions
+    const F xe = ((((((h[7] - h[8]) + h[9]) - h[10]) + h[11]) - h[12]) + h[13]) - h[14];
+    const F ye = ((((((h[7] - h[8]) - h[9]) + h[10]) + h[15]) - h[16]) + h[17]) - h[18];
+    const F ze = ((((((h[11] - h[12]) - h[13]) + h[14]) + h[15]) - h[16]) - h[17]) + h[18];
     mh[s] = vfma(F(WT(0)), h[0], vfma(F(WT(1)), sf, F(WT(7)) * se));
     const float r = a.nref[s];
-    n[s] = vfma(F(r), mh[s], F(r));
+    const F nf = vfma(F(r), mh[s], F(r));
+    n[s] = FU::density3 && s == 3 ? nf : add_scalar<NV>(r, F(r) * mh[s]);
+    const F nt = FU::total ? nf : n[s];
+    ntot = s == 0 ? nt : ntot + nt;
     jx[s] = F(r) * vfma(F(WT(1)), h[1] - h[2], F(WT(7)) * xe);
     jy[s] = F(r) * vfma(F(WT(1)), h[3] - h[4], F(WT(7)) * ye);
     jz[s] = F(r) * vfma(F(WT(1)), h[5] - h[6], F(WT(7)) * ze);
@@ -300,10 +344,9 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
     }
   }
 
-  F ntot = n[0], Jx = jx[0], Jy = jy[0], Jz = jz[0];
+  F Jx = jx[0], Jy = jy[0], Jz = jz[0];
 #pragma unroll
   for (int s = 1; s < S; ++s) {
-    ntot = ntot + n[s];
     Jx = Jx + jx[s];
     Jy = Jy + jy[s];
     Jz = Jz + jz[s];
@@ -325,9 +368,8 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
 #pragma unroll
   for (int s = 1; s < S; ++s) zn = vfma(F(a.valence[s]), n[s], zn);
   const F hzn = F(0.5f) * zn;
-  const F vbx = vfma(hzn, Ex, Jx) * inv_ntot;
-  const F vby = vfma(hzn, Ey, Jy) * inv_ntot;
-  const F vbz = vfma(hzn, Ez, Jz) * inv_ntot;
+  const F vpx = vfma(hzn, Ex, Jx), vpy = vfma(hzn, Ey, Jy), vpz = vfma(hzn, Ez, Jz);
+  const F vbx = vpx * inv_ntot, vby = vpy * inv_ntot, vbz = vpz * inv_ntot;
   // pair frequencies: the fractions x_b and x_b v_b of every species
   F px[PAIR ? S : 1], pxv[PAIR ? S : 1][3];
   if (PAIR) {
@@ -373,17 +415,17 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
           My = vfma(w, pxv[b][1], My);
           Mz = vfma(w, pxv[b][2], Mz);
         }
-        Fx = ex + (Mx - W * vx);
-        Fy = ey + (My - W * vy);
-        Fz = ez + (Mz - W * vz);
+        Fx = ex + vfma(F(0.f) - W, vx, Mx);
+        Fy = ey + vfma(F(0.f) - W, vy, My);
+        Fz = ez + vfma(F(0.f) - W, vz, Mz);
       } else {
-        Fx = vfma(F(omd), vbx - vx, ex);
-        Fy = vfma(F(omd), vby - vy, ey);
-        Fz = vfma(F(omd), vbz - vz, ez);
+        Fx = vfma(F(omd), FU::drag ? vfma(vpx, inv_ntot, F(0.f) - vx) : vbx - vx, ex);
+        Fy = vfma(F(omd), FU::drag ? vfma(vpy, inv_ntot, F(0.f) - vy) : vby - vy, ey);
+        Fz = vfma(F(omd), FU::drag ? vfma(vpz, inv_ntot, F(0.f) - vz) : vbz - vz, ez);
       }
     }
-    const F usq = vfma(usx, usx, vfma(usy, usy, usz * usz));
-    const F Fu = vfma(Fx, ux, vfma(Fy, uy, Fz * uz));
+    const F usq = vfma(usz, usz, vfma(usx, usx, usy * usy));
+    const F Fu = vfma(Fz, uz, vfma(Fx, ux, Fy * uy));
     // In deviations, d*_p = (1 - omega) d_p + [omega phi_p + g_p - omega w_p n_ref]
     // with, per weight w_p,
     //   omega phi_p + g_p - omega w_p n_ref
@@ -397,11 +439,11 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
     // the size of the deviations.
     const float inr = 1.0f / a.nref[s];
     // the per-species factors of the bracket values, once per species:
-    // even' = Ce + Ae a^2 + Be (F.c)(u.c), odd' = Do (omega a + F.c)
+    // even' = Ce + Ae a^2 + Be (F.c)(u.c), odd' = Dom a + Do F.c
     const F nin = n[s] * F(inr);
-    const F Ae = nin * F(4.5f * om), Be = nin * F(9.0f), Do = nin * F(3.0f);
-    const F Ce = vfma(nin, vfma(F(-1.5f * om), usq, F(-3.0f) * Fu), F(om) * mh[s]);
-    const F om_(om);
+    const F Ae = nin * F(4.5f * om), Be = nin * F(9.0f), Do = nin * F(3.0f), Dom = Do * F(om);
+    const F dn = mul_here(F(a.nref[s]), mh[s]), base = vfma(F(-1.5f * om), usq, F(-3.0f) * Fu);
+    const F Ce = F(inr) * (PAIR ? vfma(n[s], base, F(om) * dn) : vfma(F(om), dn, n[s] * base));
     // moving populations first; the rest population then takes
     // d*_0 = dn - sum_{p>0} d*_p over the stored (rounded) moving values,
     // i.e. h*_0 = (sum w h - sum_{p>0} w h*_p) / w_0, which holds exactly
@@ -412,15 +454,15 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
     // F.c and u.c flip sign, so each pair shares the even part and takes
     // +/- the odd part.
     const F omm(1.0f - om);
-    F mvf(0.f), mve(0.f);  // stored values summed, faces and edges
+    F moved(0.f);  // stored values, weighted and summed
     float mjx = 0.f, mjy = 0.f, mjz = 0.f;
 #pragma unroll
     for (int p = 1; p < Q; p += 2) {
       const F av = cdot<NV>(p, usx, usy, usz);
       const F fc = cdot<NV>(p, Fx, Fy, Fz);
       const F uc = cdot<NV>(p, ux, uy, uz);
-      const F even = vfma(Ae * av, av, vfma(Be * fc, uc, Ce));
-      const F odd = Do * vfma(om_, av, fc);
+      const F even = vfma(Ae, av * av, vfma(Be, fc * uc, Ce));
+      const F odd = vfma(Dom, av, Do * fc);
       F ha = vfma(omm, f[s][p].get(), even + odd), hb = vfma(omm, f[s][p + 1].get(), even - odd);
       T* pa = fout + (int64_t)(s * Q + p) * N;
       if constexpr (NV == 2) {
@@ -430,9 +472,7 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
         ha = hs.x;
         hb = hs.y;
       }
-      const F pr = ha + hb;  // same weight for p and p + 1
-      if (p <= 6) mvf = mvf + pr;
-      else mve = mve + pr;
+      moved = vfma(F(WT(p)), ha + hb, moved);  // same weight for p and p + 1
       if constexpr (SCAT) {
         // charge these stored values carry to r + c_p and r - c_p
         // (zero for a neutral species)
@@ -460,7 +500,6 @@ __device__ __forceinline__ void collide_nodes(const StepArgs& a, uint32_t i, int
         if (CZ(p)) mjz += CZ(p) * WT(p) * mj;
       }
     }
-    const F moved = vfma(F(WT(1)), mvf, F(WT(7)) * mve);
     F h0 = (mh[s] - moved) * F(INV_WT(0));
     T* p0 = fout + (int64_t)(s * Q) * N;
     if constexpr (NV == 2) Fmt<ST>::sth_sr_pair(p0, h0.a, next(0), next(1));

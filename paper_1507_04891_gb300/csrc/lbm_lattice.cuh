@@ -80,9 +80,9 @@ struct V<2> {
     else a.x = x;
   }
 };
-__device__ __forceinline__ V<1> operator+(V<1> x, V<1> y) { return x.a + y.a; }
-__device__ __forceinline__ V<1> operator-(V<1> x, V<1> y) { return x.a - y.a; }
-__device__ __forceinline__ V<1> operator*(V<1> x, V<1> y) { return x.a * y.a; }
+__device__ __forceinline__ V<1> operator+(V<1> x, V<1> y) { return __fadd_rn(x.a, y.a); }
+__device__ __forceinline__ V<1> operator-(V<1> x, V<1> y) { return __fsub_rn(x.a, y.a); }
+__device__ __forceinline__ V<1> operator*(V<1> x, V<1> y) { return __fmul_rn(x.a, y.a); }
 __device__ __forceinline__ V<1> vfma(V<1> x, V<1> y, V<1> z) { return fmaf(x.a, y.a, z.a); }
 __device__ __forceinline__ V<2> operator+(V<2> x, V<2> y) { return __fadd2_rn(x.a, y.a); }
 __device__ __forceinline__ V<2> operator-(V<2> x, V<2> y) {

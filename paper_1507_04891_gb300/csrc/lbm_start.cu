@@ -59,25 +59,25 @@ enum { ST_VALID = 0, ST_RING = 1, ST_TERMS = 2, ST_USED = 3 };
 static_assert(ST_RING == START_RING_IDX, "ring position index shared with the charge pass");
 
 // Least-squares coefficients over the first m stored differences, by one
-// warp: Gauss-Jordan elimination in FP64 (the matrix is symmetric positive
-// definite, so no pivoting) of the Gram matrix G (K x K, row-major) with a
-// relative diagonal load of 1e-10 against rounding, rows and columns from m
-// on replaced by the identity.  Lane i K + j holds entry (i, j), lane
-// K K + i the right-hand side of row i.  Returns false in every lane when a
-// pivot is not positive or a coefficient is beyond COEF_MAX (or not finite);
-// else lane K K + i returns coefficient i.  The differences of a relaxing run
-// become almost dependent, and their inner products are FP32 sums: now and
-// then the smallest pivot was rounding noise, the coefficients grew and the
-// start was so poor that the step needed a second application.  Extrapolation
-// from K = 5 differences has coefficients up to 10.  (Of 48 passes of 20
-// recorded steps at 128x64x64, 4 had such a step without the limit, none
-// with it; heavier loads of the diagonal cost multigrid cycles on the porous
-// box, 3.4 to 4.2 a step against 3.2.)
-constexpr double COEF_MAX = 16.0;
+// warp: Cholesky factorisation in FP64 of the Gram matrix G (K x K,
+// row-major) with a relative diagonal load of 1e-10 against rounding, rows
+// and columns from m on replaced by the identity.  Lane i K + j, j <= i,
+// holds entry (i, j) of the factor, lane K K + j entry j of the forward
+// substitution (the right-hand side as one more row).  Returns false in
+// every lane when a pivot is not positive or a coefficient is not finite;
+// else lane K K + i returns coefficient i.
+// The differences of a relaxing run become almost dependent, so the smallest
+// pivot is close to rounding noise and the coefficients are as good as their
+// rounding: every entry takes its terms in the order of the column loops of
+// the textbook factorisation, whatever the number of lanes.  (Gauss-Jordan
+// elimination, with or without a limit on the coefficients, gave other
+// roundings, and steps whose residual lies at the tolerance took another
+// number of applications.)
 __device__ bool solve_gram(const double* G, const double* rhs, int m, double& c) {
   const int lane = threadIdx.x & 31;
   const bool mat = lane < K * K;
-  const int i = mat ? lane / K : min(lane - K * K, K - 1), j = mat ? lane - i * K : K;
+  const int i = mat ? lane / K : K, j = mat ? lane - i * K : min(lane - K * K, K - 1);
+  const int row = mat ? i * K : K * K;  // lane of the row's entry 0
   double load = 0.0;
 #pragma unroll
   for (int q = 0; q < K; ++q)
@@ -85,21 +85,32 @@ __device__ bool solve_gram(const double* G, const double* rhs, int m, double& c)
   load = 1e-10 * load / m + 1e-300;
   double v;
   if (mat) v = (i < m && j < m) ? G[i * K + j] + (i == j ? load : 0.0) : (i == j ? 1.0 : 0.0);
-  else v = i < m ? rhs[i] : 0.0;
+  else v = j < m ? rhs[j] : 0.0;
   bool ok = true;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const double p = __shfl_sync(0xffffffffu, v, k * K + k);
     ok = ok && p > 0.0;
-    const double f = __shfl_sync(0xffffffffu, v, i * K + k) / (p > 0.0 ? p : 1.0);
-    const double row = __shfl_sync(0xffffffffu, v, mat ? k * K + j : K * K + k);
-    if (i != k) v -= f * row;
+    const double d = sqrt(p > 0.0 ? p : 1.0);
+    if (j == k) v = i == k ? d : v / d;
+    const double a = __shfl_sync(0xffffffffu, v, row + k);
+    const double b = __shfl_sync(0xffffffffu, v, j * K + k);
+    if (j > k) v = fma(-a, b, v);
   }
-  // the diagonal is left: row i's right-hand side over it
-  const double d = __shfl_sync(0xffffffffu, v, i * K + i);
-  c = v / (d != 0.0 ? d : 1.0);
-  ok = ok && (mat || fabs(c) <= COEF_MAX);
-  return __all_sync(0xffffffffu, ok);
+  // back substitution, by every lane
+  double x[K];
+#pragma unroll
+  for (int q = K - 1; q >= 0; --q) {
+    x[q] = __shfl_sync(0xffffffffu, v, K * K + q);
+#pragma unroll
+    for (int k = q + 1; k < K; ++k) x[q] = fma(-__shfl_sync(0xffffffffu, v, k * K + q), x[k], x[q]);
+    x[q] /= __shfl_sync(0xffffffffu, v, q * K + q);
+    ok = ok && isfinite(x[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < K; ++q)
+    if (j == q) c = x[q];
+  return ok;
 }
 
 // Pass 1 (one cell per thread): D_0 = s(t) - s(t-1) against D_0 and the
@@ -149,13 +160,13 @@ __global__ void __launch_bounds__(DOT_THREADS) k_start_dots(const int64_t* __res
 
 // Pass 2 (one CTA): the inner products g_j = <D_0, D_j> from the partials
 // (compensated FP32 sums in a fixed order), the coefficients over the
-// m = min(K, valid - 1) stored differences (fewer when the elimination
-// fails; the K x K elimination is the only FP64 arithmetic), the Gram
+// m = min(K, valid - 1) stored differences (fewer when the factorisation
+// fails; the K x K factorisation is the only FP64 arithmetic), the Gram
 // matrix of the next step (D_0 becomes D_1) and the bookkeeping.
-// Latency-bound: the elimination runs in one warp, an entry per lane, where
-// a thread that factorised the matrix alone spent most of the kernel
-// (porous 128^3: 18.4 -> 9.1 us; 32x8x52: 14.3 -> 5.9 us).
-constexpr int SOLVE_THREADS = 512;
+// Latency-bound: the factorisation runs in one warp, an entry per lane, where
+// a thread that factorised the matrix alone spent most of the kernel, and the
+// warps' sums of the products are joined by a warp each.
+constexpr int SOLVE_THREADS = 256;
 __global__ void __launch_bounds__(SOLVE_THREADS) k_start_solve(const float* __restrict__ part,
                                                                int nctas, double* __restrict__ gram,
                                                                float* __restrict__ coef,
@@ -199,16 +210,15 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_start_solve(const float* __re
     }
   }
   __syncthreads();
-  if (wid <= K) {  // warp j joins the warps' sums of product j
-    float h = lane < NW ? rh[wid][lane] : 0.f, l = lane < NW ? rl[wid][lane] : 0.f;
+  static_assert(NW > K, "a warp for each product");
+  if (wid <= K && lane == 0) {  // warp j joins the warps' sums of product j, in order
+    float h = 0.f, l = 0.f;
 #pragma unroll
-    for (int off = NW / 2; off > 0; off >>= 1) {
-      const float oh = __shfl_down_sync(0xffffffffu, h, off);
-      const float ol = __shfl_down_sync(0xffffffffu, l, off);
-      two_sum_add(h, l, oh);
-      l += ol;
+    for (int w = 0; w < NW; ++w) {
+      two_sum_add(h, l, rh[wid][w]);
+      l += rl[wid][w];
     }
-    if (lane == 0) g[wid] = (double)h + (double)l;
+    g[wid] = (double)h + (double)l;
   }
   __syncthreads();
   if (wid != 0) return;
