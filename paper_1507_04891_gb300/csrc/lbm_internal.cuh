@@ -158,6 +158,7 @@ struct PoissonLevel {
   int per[3];        // periodic flags
   int coarsened[3];  // 1 if this level halves that axis of the finer level
   float* e = nullptr;     // correction
+  float* e2 = nullptr;    // second buffer of the sweeps around an odd periodic extent, or NULL
   float* rhs = nullptr;   // right-hand side
   float* K = nullptr;     // [3][n] conductance to the + neighbour (levels >= 1)
   float* Dinv = nullptr;  // 1 / diagonal, 0 for an inactive cell (levels >= 1)
