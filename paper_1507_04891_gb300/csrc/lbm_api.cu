@@ -427,7 +427,10 @@ lbm_status lbm_set_walls(lbm_t* h, const uint8_t* solid, const double* sigma) {
   if (!h->links) s = dev_alloc(h, &h->links, N);
   if (s == LBM_OK && !h->wcls) s = dev_alloc(h, &h->wcls, (size_t)((N + 31) / 32));
   if (s != LBM_OK) return s;
-  LBM_CUDA_TRY(h, cudaMemcpy(sc.p, solid, N, cudaMemcpyHostToDevice));
+  // (copies in the stream of the kernels that read them: the library's stream
+  // does not wait for the default one, where a copy or a clear may still run
+  // when the call that asked for it has returned)
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(sc.p, solid, N, cudaMemcpyHostToDevice, h->st));
   h->has_walls = true;
   h->scat_on = false;  // the charge pass handles walls
   h->scat_valid = false;
@@ -438,11 +441,12 @@ lbm_status lbm_set_walls(lbm_t* h, const uint8_t* solid, const double* sigma) {
     std::vector<int64_t> wfx(N, 0);
     const double k4 = 4.0 * 3.14159265358979323846 * h->cfg.bjerrum;
     for (int64_t i = 0; i < N; ++i) wfx[i] = llrint(k4 * wd[i] * PSI_SCALE);
-    LBM_CUDA_TRY(h, cudaMemcpy(h->wallq, q.data(), N * sizeof(float), cudaMemcpyHostToDevice));
-    LBM_CUDA_TRY(h, cudaMemcpy(h->wsrc, wfx.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice));
+    LBM_CUDA_TRY(h, cudaMemcpyAsync(h->wallq, q.data(), N * sizeof(float), cudaMemcpyHostToDevice, h->st));
+    LBM_CUDA_TRY(h, cudaMemcpyAsync(h->wsrc, wfx.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice,
+                                    h->st));
+    LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));  // before the host arrays go
     if (h->cfg.bjerrum > 0.0) {
       if (!h->wallg && (s = dev_alloc(h, &h->wallg, 3 * (size_t)N)) != LBM_OK) return s;
-      LBM_CUDA_TRY(h, cudaStreamSynchronize(nullptr));  // the charges are on the device
       LBM_CUDA_TRY(h, launch_wall_gradient(h));
     }
   } else {
@@ -509,9 +513,11 @@ lbm_status lbm_set_walls(lbm_t* h, const uint8_t* solid, const double* sigma) {
       if ((s = dev_alloc(h, &P.comp_mean, P.ncomp)) != LBM_OK) return s;
       for (int64_t i = 0; i < N; ++i)
         if (lab[i] < 0) lab[i] = 0;  // wall nodes: unused
-      LBM_CUDA_TRY(h, cudaMemcpy(P.label, lab.data(), N * sizeof(int), cudaMemcpyHostToDevice));
-      LBM_CUDA_TRY(h, cudaMemcpy(P.comp_size, sizes.data(), P.ncomp * sizeof(long long),
-                                 cudaMemcpyHostToDevice));
+      LBM_CUDA_TRY(h, cudaMemcpyAsync(P.label, lab.data(), N * sizeof(int), cudaMemcpyHostToDevice,
+                                      h->st));
+      LBM_CUDA_TRY(h, cudaMemcpyAsync(P.comp_size, sizes.data(), P.ncomp * sizeof(long long),
+                                      cudaMemcpyHostToDevice, h->st));
+      LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));
     }
     s = poisson_setup(h, solid);
     if (s != LBM_OK) return s;
@@ -554,8 +560,8 @@ lbm_status lbm_set_species(lbm_t* h, int s, double mass, double valence,
   if (cudaMalloc(&sc.p, bytes) != cudaSuccess) return fail(h, LBM_ENOMEM, "scratch allocation failed");
   double* dn = (double*)sc.p;
   double* du = u0 ? dn + N : nullptr;
-  LBM_CUDA_TRY(h, cudaMemcpy(dn, n0, N * sizeof(double), cudaMemcpyHostToDevice));
-  if (u0) LBM_CUDA_TRY(h, cudaMemcpy(du, u0, 3 * N * sizeof(double), cudaMemcpyHostToDevice));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(dn, n0, N * sizeof(double), cudaMemcpyHostToDevice, h->st));
+  if (u0) LBM_CUDA_TRY(h, cudaMemcpyAsync(du, u0, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->st));
   LBM_CUDA_TRY(h, launch_init_species(h, s, dn, du));
   LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));
   return species_done(h, s, mass, valence);
@@ -1031,7 +1037,11 @@ lbm_status lbm_set_plane_omega_drag(lbm_t* h, const double* omega) {
     lbm_status s = dev_alloc(h, &h->omega_drag_z, nz);
     if (s != LBM_OK) return s;
   }
-  LBM_CUDA_TRY(h, cudaMemcpy(h->omega_drag_z, w.data(), nz * sizeof(float), cudaMemcpyHostToDevice));
+  // after the steps that are queued
+  LBM_CUDA_TRY(h, own_stream(h));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(h->omega_drag_z, w.data(), nz * sizeof(float), cudaMemcpyHostToDevice,
+                                  h->st));
+  LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));
   spectral_graph_free(h);
   return LBM_OK;
 }

@@ -710,9 +710,9 @@ lbm_status nn_init(lbm_t* h, int hidden, uint64_t seed) {
   const float a1 = sqrtf(3.f / (2.f * 27.f)), a2 = 0.1f * sqrtf(3.f / (hidden * 27.f));
   for (int k = 0; k < hidden * 2 * 27; ++k) p[k] = a1 * U(rng);
   for (int k = 0; k < hidden * 27; ++k) p[hidden * 2 * 27 + hidden + k] = a2 * U(rng);
-  LBM_CUDA_TRY(h, cudaMemcpy(n->p, p.data(), n->np * sizeof(float), cudaMemcpyHostToDevice));
-  LBM_CUDA_TRY(h, cudaMemset(n->m, 0, n->np * sizeof(float)));
-  LBM_CUDA_TRY(h, cudaMemset(n->v, 0, n->np * sizeof(float)));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(n->p, p.data(), n->np * sizeof(float), cudaMemcpyHostToDevice, h->st));
+  LBM_CUDA_TRY(h, cudaMemsetAsync(n->m, 0, n->np * sizeof(float), h->st));
+  LBM_CUDA_TRY(h, cudaMemsetAsync(n->v, 0, n->np * sizeof(float), h->st));
   k_to_half<<<nb(n->np, 256), 256, 0, h->st>>>(n->p, n->ph, n->np);
   LBM_CUDA_TRY(h, cudaGetLastError());
   LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));
@@ -923,9 +923,12 @@ lbm_status nn_params(lbm_t* h, float* get, const float* set, int* np) {
     return LBM_EINVAL;
   }
   if (np) *np = n->np;
-  if (get) LBM_CUDA_TRY(h, cudaMemcpy(get, n->p, n->np * sizeof(float), cudaMemcpyDeviceToHost));
+  if (get) {
+    LBM_CUDA_TRY(h, cudaMemcpyAsync(get, n->p, n->np * sizeof(float), cudaMemcpyDeviceToHost, h->st));
+    LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));
+  }
   if (set) {
-    LBM_CUDA_TRY(h, cudaMemcpy(n->p, set, n->np * sizeof(float), cudaMemcpyHostToDevice));
+    LBM_CUDA_TRY(h, cudaMemcpyAsync(n->p, set, n->np * sizeof(float), cudaMemcpyHostToDevice, h->st));
     n->hp_stale = true;
     k_to_half<<<nb(n->np, 256), 256, 0, h->st>>>(n->p, n->ph, n->np);
     LBM_CUDA_TRY(h, cudaGetLastError());

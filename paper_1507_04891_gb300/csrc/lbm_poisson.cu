@@ -1606,10 +1606,10 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
   }
   // wall cells and pad cells are never read; cleared once so that no
   // uninitialised value is ever visible
-  cudaMemset(L0.e, 0, split * sizeof(float));
-  if (L0.e2) cudaMemset(L0.e2, 0, split * sizeof(float));
-  cudaMemset(L0.rhs, 0, split * sizeof(float));
   P.lev.push_back(L0);
+  LBM_CUDA_TRY(h, cudaMemsetAsync(L0.e, 0, split * sizeof(float), h->st));
+  if (L0.e2) LBM_CUDA_TRY(h, cudaMemsetAsync(L0.e2, 0, split * sizeof(float), h->st));
+  LBM_CUDA_TRY(h, cudaMemsetAsync(L0.rhs, 0, split * sizeof(float), h->st));
   cudaFree(P.face);
   P.face = nullptr;
   if (h->has_walls) {
@@ -1617,7 +1617,8 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
       h->err = "Poisson face mask allocation failed";
       return LBM_ENOMEM;
     }
-    cudaMemset(P.face, (int)FACE_SOLID, split);
+    // (before k_face_mask, so in its stream)
+    LBM_CUDA_TRY(h, cudaMemsetAsync(P.face, (int)FACE_SOLID, split, h->st));
     const Box b = make_box(h);
     k_face_mask<<<nblocks(L0.n, 256), 256, 0, h->st>>>(h->links, b, (uint32_t)L0.n, P.face);
     LBM_CUDA_TRY(h, cudaGetLastError());
@@ -1711,9 +1712,10 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
       P.lev.push_back(L);
       return LBM_ENOMEM;
     }
-    cudaMemcpy(L.K, Kc.data(), 3 * n * sizeof(float), cudaMemcpyHostToDevice);
-    cudaMemcpy(L.Dinv, Dv.data(), n * sizeof(float), cudaMemcpyHostToDevice);
     P.lev.push_back(L);
+    LBM_CUDA_TRY(h, cudaMemcpyAsync(L.K, Kc.data(), 3 * n * sizeof(float), cudaMemcpyHostToDevice, h->st));
+    LBM_CUDA_TRY(h, cudaMemcpyAsync(L.Dinv, Dv.data(), n * sizeof(float), cudaMemcpyHostToDevice, h->st));
+    LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));  // before the host arrays go
     Kh.swap(Kc);
     act.swap(ac);
     lx = Lx;

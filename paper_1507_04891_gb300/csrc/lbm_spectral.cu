@@ -1131,12 +1131,13 @@ lbm_status spectral_setup(lbm_t* h, const uint8_t* solid) {
   for (int k = 0; k <= nx / 2; ++k) lam.push_back(eig(k, nx));
   for (int k = 0; k < ny; ++k) lam.push_back(eig(k, ny));
   for (int k = 0; k < nz; ++k) lam.push_back(eig(k, nz));
-  LBM_CUDA_TRY(h, cudaMemset(s->mean_z, 0, nz * sizeof(long long)));
-  LBM_CUDA_TRY(h, cudaMemcpy(s->planes, planes.data(), planes.size() * sizeof(int), cudaMemcpyHostToDevice));
-  LBM_CUDA_TRY(h, cudaMemcpy(s->runs, runs.data(), runs.size() * sizeof(Run), cudaMemcpyHostToDevice));
-  LBM_CUDA_TRY(h, cudaMemcpy(s->plane_fluid, pf.data(), nz, cudaMemcpyHostToDevice));
-  LBM_CUDA_TRY(h, cudaMemcpy(s->tw, tw.data(), ntw * sizeof(float2), cudaMemcpyHostToDevice));
-  LBM_CUDA_TRY(h, cudaMemcpy(s->lam, lam.data(), nlam * sizeof(float), cudaMemcpyHostToDevice));
+  LBM_CUDA_TRY(h, cudaMemsetAsync(s->mean_z, 0, nz * sizeof(long long), h->st));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(s->planes, planes.data(), planes.size() * sizeof(int), cudaMemcpyHostToDevice, h->st));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(s->runs, runs.data(), runs.size() * sizeof(Run), cudaMemcpyHostToDevice, h->st));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(s->plane_fluid, pf.data(), nz, cudaMemcpyHostToDevice, h->st));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(s->tw, tw.data(), ntw * sizeof(float2), cudaMemcpyHostToDevice, h->st));
+  LBM_CUDA_TRY(h, cudaMemcpyAsync(s->lam, lam.data(), nlam * sizeof(float), cudaMemcpyHostToDevice, h->st));
+  LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));  // before the host arrays go
   int optin = 0;
   LBM_CUDA_TRY(h, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
   const int lgz = ilog2(nz);
@@ -1176,7 +1177,6 @@ lbm_status spectral_setup(lbm_t* h, const uint8_t* solid) {
       h->err = "spectral Poisson allocation failed";
       return LBM_ENOMEM;
     }
-    LBM_CUDA_TRY(h, cudaStreamSynchronize(nullptr));  // the eigenvalues are on the device
     k_ztable<<<nblk(s->mxy, 128), 128, 0, h->st>>>(s->ztab, s->qtab, lmax, cyclic, args_of(s));
     LBM_CUDA_TRY(h, cudaGetLastError());
   }
@@ -1860,8 +1860,9 @@ lbm_status spectral_graph_steps(lbm_t* h, int nsteps) {
     GraphStatus z = {};
     z.step = (uint32_t)h->tstep;
     z.start_mant = 1.0;
-    cudaMemcpy(p, &z, sizeof z, cudaMemcpyHostToDevice);
     h->gstatus = p;
+    LBM_CUDA_TRY(h, cudaMemcpyAsync(p, &z, sizeof z, cudaMemcpyHostToDevice, h->st));
+    LBM_CUDA_TRY(h, cudaStreamSynchronize(h->st));
     if (cudaMallocHost(&h->hstatus, sizeof(GraphStatus)) != cudaSuccess) {
       h->err = "pinned allocation failed";
       return LBM_ENOMEM;

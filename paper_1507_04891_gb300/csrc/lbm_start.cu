@@ -504,7 +504,7 @@ lbm_status start_setup(lbm_t* h) {
       cudaGetLastError();
       return false;
     }
-    return cudaMemset(*p, 0, bytes) == cudaSuccess;
+    return cudaMemsetAsync(*p, 0, bytes, h->st) == cudaSuccess;
   };
   const bool ok = al((void**)&H.s_prev, N * sizeof(int64_t)) &&
                   al((void**)&H.psi_prev, N * sizeof(int64_t)) &&
