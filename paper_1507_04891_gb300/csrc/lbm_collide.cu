@@ -32,9 +32,9 @@ namespace {
 //      opposite direction when r + c_p is a wall node), so the sums of the
 //      stored values give the next state's species masses, and the stored
 //      values signed by the direction they are pulled in give its momentum.
-//      Per CTA: the deviation sums (FP32 within a warp, FP64 across warps)
-//      and a count of nodes whose density entering the step was not finite
-//      and positive, written to a[blockIdx.x * DIAG_NQ + k].
+//      Per CTA: the deviation sums (FP32 over 32 nodes, FP64 over more) and
+//      a count of densities (of a node and species) entering the step that
+//      were not finite and positive, written to a[blockIdx.x * DIAG_NQ + k].
 // ---------------------------------------------------------------------------
 // NV nodes per thread (V<NV>, lbm_lattice.cuh): one in FP32, two consecutive
 // x nodes in the 16-bit formats when nx is even.  The 16-bit kernel is bound
@@ -691,20 +691,23 @@ __global__ void __launch_bounds__(256) __maxnreg__((collide_maxnreg<S, NV>()))
   if (DIAG) {
     float v[DIAG_NQ];
     diag_quantities<S>(a, q, v);
-    __shared__ float red[8][DIAG_NQ];
+    // 32 nodes are added in FP32, by the LANES lanes that hold them, the rest
+    // in FP64
+    constexpr int LANES = 32 / NV;
+    __shared__ float red[256 / LANES][DIAG_NQ];
 #pragma unroll
     for (int k = 0; k < DIAG_NQ; ++k) {
       if (k >= S && k < MAX_SPECIES) continue;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v[k];
+      for (int off = LANES / 2; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
+      if (threadIdx.x % LANES == 0) red[threadIdx.x / LANES][k] = v[k];
     }
     __syncthreads();
     if (threadIdx.x < DIAG_NQ) {
       const int k = threadIdx.x;
       double tot = 0.0;
       if (k < S || k >= MAX_SPECIES)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += (double)red[w][k];
+        for (int w = 0; w < (int)blockDim.x / LANES; ++w) tot += (double)red[w][k];
       a.diag[(int64_t)blockIdx.x * DIAG_NQ + k] = tot;
     }
   }
