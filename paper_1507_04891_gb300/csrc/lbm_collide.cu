@@ -539,14 +539,18 @@ __device__ __forceinline__ void diag_quantities(const StepArgs& a, const Sums<S>
 // Registers: up to 128 per thread (16 warps per SM), 255 for four species.
 // Two nodes per thread of three species: 168 (12 warps); ternary 128^3 FP16
 // took 110 us with 168 in ncu, 123 with 128 (spills), 108 against 102 with
-// 144; 64 slits 271 us with 168, 331 with 200, 322 with 255.
-template <int S, int NV>
+// 144; 64 slits 271 us with 168, 331 with 200, 322 with 255.  One node per
+// thread of three species in 16 bits (odd nx), bound by instruction issue
+// and not by HBM: 92, 20 warps in CTAs of 128 threads (127x128x128 FP16:
+// 120 us a launch, 124.5 with 128, 126.7 with 96, 120.6 with 88; beside
+// wall planes 128, 137 with 128; neutral 115, 118.5; BF16 120, 124.5).
+template <int S, int NV, int ST>
 constexpr int collide_maxnreg() {
-  return S >= 4 ? 255 : (S == 3 && NV == 2 ? 168 : 128);
+  return S >= 4 ? 255 : (S < 3 ? 128 : (NV == 2 ? 168 : (ST == LBM_FP32 ? 128 : 92)));
 }
 
 template <int S, int NV, bool WALLS, bool CHARGED, int ST, bool DIAG, bool PAIR, bool SCAT>
-__global__ void __launch_bounds__(256) __maxnreg__((collide_maxnreg<S, NV>()))
+__global__ void __launch_bounds__(256) __maxnreg__((collide_maxnreg<S, NV, ST>()))
     k_stream_collide(const StepArgs a) {
   using T = typename Fmt<ST>::T;
   // neutral lattices, whose launch need not wait for the previous kernel to
