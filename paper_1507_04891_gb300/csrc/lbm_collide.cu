@@ -723,11 +723,12 @@ cudaError_t launch_one(const StepArgs& a, cudaStream_t st, int threads, int64_t*
   *ctas = nblocks(a.N / NV, threads);
   // A step of a neutral lattice is this one kernel.  Programmatic
   // serialisation brings up the next step's CTAs beside the last ones of this
-  // step, which shortens small boxes (32^3 binary, 100 steps: 248 -> 231 us);
-  // grids of more than about one wave gain nothing (97x61x45, four species:
-  // 598 against 601 us) and keep the plain launch.
-  constexpr int64_t ONE_WAVE = 4 * 152;
-  if (!C && *ctas <= ONE_WAVE) {
+  // step, which shortens small boxes (32^3 binary, 256 CTAs, 100 steps: 248 ->
+  // 231 us); grids of more than one wave gain nothing (97x61x45, four
+  // species, about seven waves: 598 against 601 us) and keep the plain launch.
+  // One wave: what the registers of an SM (65536) hold at the kernel's cap.
+  const int64_t one_wave = (int64_t)a.sms * (65536 / (collide_maxnreg<S, NV, ST>() * threads));
+  if (!C && *ctas <= one_wave) {
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;

@@ -118,6 +118,7 @@ struct StepArgs {
   const float* wallq;      // face charge share of each wall node; may be NULL
   const float* wallg;      // wall part of the potential's gradient, [3][N]; may be NULL
   int nx, ny, nz;
+  int sms;                 // SMs of the device (for the launch)
   int64_t N;
   float omega_visc, omega_drag;
   const float* omega_drag_z;  // per z-plane drag frequency (stacked instances) or NULL

@@ -901,6 +901,7 @@ StepArgs step_args(lbm_t* h) {
   a.nx = h->cfg.nx;
   a.ny = h->cfg.ny;
   a.nz = h->cfg.nz;
+  a.sms = h->grid_cap / 8;
   a.N = h->N;
   a.omega_visc = (float)h->cfg.omega_visc;
   a.omega_drag = (float)h->cfg.omega_drag;
