@@ -147,19 +147,6 @@ struct Fmt<LBM_FP32> {
     *pb = hb;
     return make_float2(ha, hb);
   }
-  // the same for two consecutive nodes (pa, pb even): ha, hb become the
-  // stored values
-  static __device__ __forceinline__ float2 ldh2(const T* p) {
-    return *reinterpret_cast<const float2*>(p);
-  }
-  static __device__ __forceinline__ void sth_sr22(T* pa, float2& ha, T* pb, float2& hb, uint32_t,
-                                                  uint32_t) {
-    *reinterpret_cast<float2*>(pa) = ha;
-    *reinterpret_cast<float2*>(pb) = hb;
-  }
-  static __device__ __forceinline__ void sth_sr_pair(T* p, float2& h, uint32_t, uint32_t) {
-    *reinterpret_cast<float2*>(p) = h;
-  }
 };
 
 // Two values rounded stochastically into a packed 16-bit pair by the
@@ -205,12 +192,9 @@ struct Fmt<LBM_FP16_SHIFT> {
     const float2 r = __half22float2(*reinterpret_cast<const __half2*>(&v));
     return make_float2(r.y, r.x);  // ha sits in the upper half
   }
-  static __device__ __forceinline__ float2 ldh2(const T* p) {
-    const uint32_t v = *reinterpret_cast<const uint32_t*>(p);
-    return unpack(v);
-  }
-  // two consecutive nodes, random bits r0, r1 of their own (the same
-  // roundings as sth_sr2 of each): the halves regrouped per direction
+  // two consecutive nodes (pa, pb even), random bits r0, r1 of their own (the
+  // same roundings as sth_sr2 of each): the halves regrouped per direction;
+  // ha, hb become the stored values
   static __device__ __forceinline__ void sth_sr22(T* pa, float2& ha, T* pb, float2& hb, uint32_t r0,
                                                   uint32_t r1) {
     const uint32_t v0 = cvt_rs_f16x2(ha.x, hb.x, r0), v1 = cvt_rs_f16x2(ha.y, hb.y, r1);
@@ -254,12 +238,9 @@ struct Fmt<LBM_BF16_SHIFT> {
     *reinterpret_cast<unsigned short*>(pb) = (unsigned short)(v & 0xFFFFu);
     return make_float2(__uint_as_float(v & 0xFFFF0000u), __uint_as_float(v << 16));
   }
-  static __device__ __forceinline__ float2 ldh2(const T* p) {
-    const uint32_t v = *reinterpret_cast<const uint32_t*>(p);
-    return unpack(v);
-  }
-  // two consecutive nodes, random bits r0, r1 of their own (the same
-  // roundings as sth_sr2 of each): the halves regrouped per direction
+  // two consecutive nodes (pa, pb even), random bits r0, r1 of their own (the
+  // same roundings as sth_sr2 of each): the halves regrouped per direction;
+  // ha, hb become the stored values
   static __device__ __forceinline__ void sth_sr22(T* pa, float2& ha, T* pb, float2& hb, uint32_t r0,
                                                   uint32_t r1) {
     const uint32_t v0 = cvt_rs_bf16x2(ha.x, hb.x, r0), v1 = cvt_rs_bf16x2(ha.y, hb.y, r1);
