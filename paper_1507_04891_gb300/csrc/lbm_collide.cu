@@ -80,22 +80,6 @@ struct Scat {
   }
 };
 
-// Nearest fixed-point integer of a float below 2^63: the part above 2^32
-// (rounded, so that the rest is exact in FP32 and signed) and the rest, each
-// by the 32-bit conversion; a rest of 2^31, which the conversion saturates to
-// 2^31 - 1 (no other rest gives that: FP32 steps by 128 there), gets its unit
-// back.
-// Ten instructions; f32_to_i64_rn's shifts of 64-bit words took about
-// three times as many, and the scatter converts 9 to 14 sums per node.
-// With the 32-bit node offsets and the reciprocal of vrcp the kernel with the
-// scatter went from 1.30e8 to 1.06e8 warp instructions at 128^3, 178.6 ->
-// 155.0 us in ncu, 180 -> 166 in the step.
-__device__ __forceinline__ unsigned long long scat_fixed(float c) {
-  const int hi = __float2int_rn(c * 2.3283064365386963e-10f);
-  const int lo = __float2int_rn(fmaf(-4294967296.0f, (float)hi, c));
-  return (unsigned long long)(((long long)hi << 32) + (long long)lo + (lo == 0x7fffffff ? 1 : 0));
-}
-
 // A warp holds 32 consecutive nodes of one x row (nx is a multiple of 32).
 // Per target group (dy, dz) a lane adds the contributions that reach its own
 // x: its own ones with c_x = 0, those of lane - 1 with c_x = +1 and of
