@@ -42,8 +42,8 @@ namespace {
 // HBM: with two nodes the arithmetic issues packed FP32 instructions, the
 // populations wait in registers as packed pairs, addresses are formed once
 // per pair and directions without an x component move as one word
-// (ternary 128^3, FP16: 1.10e8 -> 6.4e7 warp instructions, 122.7 -> 101.7 us
-// in ncu; 64 slits of 32x32 342 -> 271 us in the step).  In FP32 two nodes
+// (ternary 128^3, FP16: 1.10e8 -> 6.7e7 warp instructions, 122.6 -> 106 us a
+// launch; with wall planes 153 -> 124 us).  In FP32 two nodes
 // per thread need over 200 registers: 8 warps per SM instead of 16, 234 us
 // against 180, and a form that landed the next tile in shared memory behind
 // the arithmetic 223 us, so FP32 keeps one node.
@@ -209,7 +209,12 @@ __device__ __forceinline__ const T* pop_at(const void* base, int64_t plane, uint
 // each an exact integer difference, rounded once (a step of psi up to 2^11
 // per face).  At a wall face the node's own value takes the neighbour's
 // place and the Neumann value of the surface-charge condition is in the wall
-// part w (k_wall_gradient).
+// part w (k_wall_gradient).  The conversions issue on the FP64 pipe, six per
+// node: the difference over two nodes, rounded once, would need three (128^3
+// with wall planes 165 -> 155 us a launch), but rounds otherwise and wraps at
+// half the step; joining two exact 32-bit pieces instead (157 us there) was
+// slower without walls (with the scatter 166 against 162 us, FP16 114
+// against 106).
 template <bool WALLS>
 __device__ __forceinline__ float axis_gradient(int64_t c, int64_t m, int64_t p, uint32_t wm, uint32_t wp,
                                                float w) {
@@ -521,9 +526,9 @@ __device__ __forceinline__ void diag_quantities(const StepArgs& a, const Sums<S>
 }
 
 // Registers: up to 128 per thread (16 warps per SM), 255 for four species.
-// Two nodes per thread of three species: 168 (12 warps); ternary 128^3 FP16
-// took 110 us with 168 in ncu, 123 with 128 (spills), 108 against 102 with
-// 144; 64 slits 271 us with 168, 331 with 200, 322 with 255.  One node per
+// Two nodes per thread of three species: 168 (12 warps); in a sweep ternary
+// 128^3 FP16 took 102 us with 168 in ncu, 123 with 128 (spills), 108 with 144;
+// 64 slits 271 us with 168, 331 with 200, 322 with 255.  One node per
 // thread of three species in 16 bits (odd nx), bound by instruction issue
 // and not by HBM: 92, 20 warps in CTAs of 128 threads (127x128x128 FP16:
 // 120 us a launch, 124.5 with 128, 126.7 with 96, 120.6 with 88; beside

@@ -287,7 +287,7 @@ struct lbm {
   // step counter advanced by the charge path while graph steps are captured
   uint32_t* charge_step = nullptr;
   const int* collide_skip = nullptr;  // skip flag of the stream/collide being captured
-  // extra duties of the start's bookkeeping kernel while a step graph is
+  // extra duties of the start's bookkeeping (start_mark) while a step graph is
   // captured: the speculation flag and the first norm slot to clear
   int* mark_skip_out = nullptr;
   const int* mark_prev_iters = nullptr;  // the previous step's applications (graph status)

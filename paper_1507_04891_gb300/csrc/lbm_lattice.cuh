@@ -388,8 +388,8 @@ __device__ __forceinline__ void psi_gradient(const StepArgs& a, uint32_t i,
 // Ten instructions; f32_to_i64_rn's shifts of 64-bit words took about
 // three times as many, and the scatter converts 9 to 14 sums per node.
 // With the 32-bit node offsets and the reciprocal of vrcp the kernel with the
-// scatter went from 1.30e8 to 1.06e8 warp instructions at 128^3, 178.6 ->
-// 155.0 us in ncu, 180 -> 166 in the step.
+// scatter went from 1.30e8 to 1.13e8 warp instructions at 128^3, 178 -> 162
+// us a launch, 180 -> 165 in the step.
 __device__ __forceinline__ unsigned long long scat_fixed(float c) {
   const int hi = __float2int_rn(c * 2.3283064365386963e-10f);
   const int lo = __float2int_rn(fmaf(-4294967296.0f, (float)hi, c));

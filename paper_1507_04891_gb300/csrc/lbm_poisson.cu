@@ -809,7 +809,10 @@ __device__ __forceinline__ bool odd_end(const CL& l, int x, int y, int z) {
 // which they form themselves.  (With old values on both sides the level's
 // short last cells, tightly bound to the first ones, are smoothed badly: a
 // cycle on 90x50x75 would reduce the residual 4.9 times instead of 5.6, on
-// 33x18x21 5.6 instead of 7.5 times.)  No load waits for another.
+// 33x18x21 5.6 instead of 7.5 times.)  No load waits for another: five steps
+// on 90x50x75 take 2147 us, 2267 with the loads behind branches, 2489 with old
+// values everywhere; a barrier between the odd ends and the others in shared
+// memory instead of forming values twice made k_sub_cycle 44 us, this 36.
 __device__ __forceinline__ float gs_odd(const float* x, const float* rhs, const float* K,
                                         const float* Dinv, const CL& l, uint32_t c, int xx, int yy,
                                         int zz) {
@@ -1322,7 +1325,7 @@ __device__ __forceinline__ void bottom_sweeps(float* e, const float* rhs, const 
 // Latency- and issue-bound (one SM): the places of a thread's cells are found
 // once per smoothing call instead of once per half-sweep, a coarse cell's
 // children are restricted by eight lanes, and one warp does the coarsest
-// level (bottom_sweeps).  16^3 cells and below: 58.2 us in ncu, now 41.1.
+// level (bottom_sweeps).  16^3 cells and below: 58.2 us in ncu, now 40.9.
 // ODD: a level of more than 64 cells has an odd periodic extent (gs_odd, whose
 // registers the other instance does without).
 template <bool ODD>
@@ -1635,7 +1638,7 @@ lbm_status poisson_setup(lbm_t* h, const uint8_t* solid) {
   // An odd extent halves too: its last coarse cell keeps one child.  (While
   // only even extents halved, a box of 90x50x75 stopped at 45x25x75 cells and
   // 50 sweeps over them per cycle were the coarse solve, 100 launches: a step
-  // of a ternary mixture took 2.4 to 4.8 ms; now 0.41 ms.)  Short axes halve
+  // of a ternary mixture took 2.4 to 4.8 ms; now 0.43 ms.)  Short axes halve
   // down to one cell, below the finest level also from two: where they
   // stopped at two or three, the cells of a long box grew ever longer and a
   // cycle smoothed little (to 1e-9, 40x5x3: 64 cycles, now 12; 64x3x3: 202,

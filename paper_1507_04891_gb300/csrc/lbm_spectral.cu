@@ -1468,9 +1468,9 @@ __global__ void k_loop_seed(const GraphStatus* st, cudaGraphConditionalHandle co
 // usually needs more applications, and the speculative stream/collide would
 // be discarded; then the stream/collide runs once, after the loop.
 // The step after one that needed more than the k baked applications does
-// not speculate either (such steps come in runs; see k_start_mark).  This
-// kernel decides when the start from the history is off; otherwise the
-// start's bookkeeping kernel does.
+// not speculate either (such steps come in runs; see start_mark).  This
+// kernel decides when the start from the history is off; otherwise start_mark
+// does.
 __global__ void k_spec_decide(const int* __restrict__ start_terms, GraphStatus* st, int k) {
   st->spec_skip = ((start_terms && *start_terms < START_FULL_TERMS) || st->iters > k) ? 1 : 0;
 }

@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(DOT_THREADS) k_start_dots(const int64_t* __res
 // matrix of the next step (D_0 becomes D_1) and the bookkeeping.
 // Latency-bound: the factorisation runs in one warp, an entry per lane, where
 // a thread that factorised the matrix alone spent most of the kernel, and the
-// warps' sums of the products are joined by a warp each.
+// warps' sums of the products are joined by a warp each (porous 128^3: 18.4 ->
+// 14.8 us in ncu, most of it the chain of FP64 roots and divisions).
 constexpr int SOLVE_THREADS = 256;
 __global__ void __launch_bounds__(SOLVE_THREADS) k_start_solve(const float* __restrict__ part,
                                                                int nctas, double* __restrict__ gram,
